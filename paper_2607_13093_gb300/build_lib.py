@@ -3,7 +3,9 @@
 Each translation unit compiles in parallel to an object file under _lib/;
 the objects link into _lib/libsph.so against the shared CUDA runtime (the
 same libcudart the process already uses for PyTorch).  A source newer than
-its object, or a changed header, triggers a rebuild of that unit.
+its object, or a changed header, triggers a rebuild of that unit.  Beside it
+g++ builds _lib/py_fast.so, the binding's native argument marshalling,
+against the installed PyTorch.
 """
 from __future__ import annotations
 
@@ -12,6 +14,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -19,6 +22,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OUT = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUT, "libsph.so")
+FAST = os.path.join(OUT, "py_fast.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
@@ -50,6 +54,18 @@ def _stale(obj: str, src: str, newest_header: float) -> bool:
     return os.path.getmtime(src) > t or newest_header > t
 
 
+def _fast_cmd(src: str):
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    inc, lib = os.path.join(root, "include"), os.path.join(root, "lib")
+    abi = int(getattr(torch._C, "_GLIBCXX_USE_CXX11_ABI", True))
+    return [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-fPIC", "-shared",
+            f"-D_GLIBCXX_USE_CXX11_ABI={abi}", "-I", INCLUDE,
+            "-I", sysconfig.get_paths()["include"], "-I", inc,
+            "-I", os.path.join(inc, "torch", "csrc", "api", "include"), src, "-o", FAST,
+            "-L", lib, f"-Wl,-rpath,{lib}", "-lc10", "-ltorch_cpu", "-ltorch_python", "-ldl"]
+
+
 def build(verbose: bool = False, force: bool = False, extra_flags=()) -> str:
     """Compile every csrc/*.cu and link _lib/libsph.so; returns its path."""
     os.makedirs(OUT, exist_ok=True)
@@ -65,6 +81,11 @@ def build(verbose: bool = False, force: bool = False, extra_flags=()) -> str:
             cmd = [cc, *ARCH, *NVCC_FLAGS, *extra_flags, "-I", INCLUDE,
                    "-I", CSRC, "-c", s, "-o", o]
             jobs.append((s, cmd))
+
+    relink = bool(jobs) or force or not os.path.exists(LIB)
+    fast_src = os.path.join(CSRC, "py_fast.cpp")
+    if force or _stale(FAST, fast_src, newest_header):
+        jobs.append((fast_src, _fast_cmd(fast_src)))
 
     def run(job):
         src, cmd = job
@@ -82,8 +103,8 @@ def build(verbose: bool = False, force: bool = False, extra_flags=()) -> str:
                 failed.append((src, r.stdout + r.stderr))
     if failed:
         msg = "\n".join(f"{s}:\n{out}" for s, out in failed)
-        raise RuntimeError("nvcc failed:\n" + msg)
-    if jobs or force or not os.path.exists(LIB):
+        raise RuntimeError("compiling failed:\n" + msg)
+    if relink:
         cmd = [cc, *ARCH, "-shared", "-cudart", "shared", "-o", LIB, *objs]
         if verbose:
             print(" ".join(cmd), flush=True)

@@ -4,6 +4,9 @@ Argument marshalling only: tensors are passed as device pointers with their
 leading dimensions, PyTorch supplies the device memory and the stream, and
 every step of the computation runs in the library's CUDA kernels.  There is
 no fallback: if the library is not built, importing this module raises.
+The hot-path calls whose outputs are given are marshalled natively
+(csrc/py_fast.cpp); what that does not take goes through the Python checks
+below, which decide what is accepted.
 
 Functions carry the C names (sph_partial_logits, sph_fuse_sample,
 sph_verify_draft, ...) and take torch tensors; `Context` bundles a context
@@ -125,6 +128,43 @@ def _load() -> ctypes.CDLL:
 
 lib = _load()
 LIB_PATH = _LIB_PATH
+
+
+def _load_fast():
+    import importlib.util
+    path = os.path.join(os.path.dirname(_LIB_PATH), "py_fast.so")
+    if not os.path.exists(path):
+        raise RuntimeError(
+            f"py_fast.so is not built ({path}); run "
+            "`python -c 'import __graft_entry__ as g; g.build()'` first")
+    spec = importlib.util.spec_from_file_location("py_fast", path)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    mod.bind(_LIB_PATH)
+    return mod
+
+
+_fast = _load_fast()
+_NOT_TAKEN = -1000       # the native marshalling leaves the call to Python
+
+
+def _word(ctx):
+    """The handle as an integer; None (not taken natively) if it is not one."""
+    return ctx.value if type(ctx) is ctypes.c_void_p else None
+
+
+def _refused(ctx, r: int):
+    """A native call's negative outcome: an error of the library raises;
+    returns where the call was not made."""
+    if r != _NOT_TAKEN:
+        _check(ctx, -1 - r)
+
+
+try:
+    _raw_stream = torch._C._cuda_getCurrentRawStream
+except AttributeError:
+    def _raw_stream(device):
+        return torch.cuda.current_stream(device).cuda_stream
 
 
 class SphError(RuntimeError):
@@ -270,6 +310,12 @@ def sph_partial_logits(ctx, h_cloud, W_h, *, keep_ids=None, clip=30.0,
     """Cloud call.  Returns (codes int8 [R, n], row_scale fp32 [R],
     payload_bytes).  h_cloud fp32 [R, d_h] (any row stride); W_h bf16 or
     float8_e4m3fn [V, d_h]."""
+    if codes is not None and row_scale is not None:
+        r = _fast.partial_logits(_word(ctx), h_cloud, W_h, keep_ids, clip, w_row_scale, bias,
+                                 act_mode, codes, row_scale, partial_out)
+        if r >= 0:
+            return codes, row_scale, r
+        _refused(ctx, r)
     _need(h_cloud, torch.float32, "h_cloud")
     if W_h.dtype == torch.bfloat16:
         wdt = SPH_DTYPE_BF16
@@ -368,6 +414,12 @@ def sph_fuse_sample(ctx, codes, row_scale, h_local, W_l, *, keep_ids=None,
     """Endpoint call.  Returns tokens int32 [R] (vocabulary ids); with
     draw=False only z is computed (into fused_logits_out, required) and the
     call returns None."""
+    if (tokens is not None) if draw else (tokens is None and fused_logits_out is not None):
+        r = _fast.fuse_sample(_word(ctx), codes, row_scale, h_local, W_l, keep_ids, temperature,
+                              seed, offset, tokens, fused_logits_out)
+        if r >= 0:
+            return tokens
+        _refused(ctx, r)
     _need(codes, torch.int8, "codes")
     _need(row_scale, torch.float32, "row_scale")
     _need(h_local, torch.float32, "h_local")
@@ -402,6 +454,14 @@ def sph_split_step(ctx, h, d_l: int, W_h, W_l, *, keep_ids=None, clip=30.0,
     the endpoint's part, h[:, d_l:] the cloud's) to tokens.  Returns
     (codes, scales, tokens, payload_bytes): the payload that would cross,
     chunk-major (int8 [R * n] flat, fp32 [nchunk * R])."""
+    if codes is not None and scales is not None and tokens is not None \
+            and fused_logits_out is None:
+        r = _fast.split_step(_word(ctx), h, d_l, W_h, W_l, keep_ids, clip, w_row_scale, bias,
+                             act_mode, temperature, seed, offset, chunk, endpoint_stream or 0,
+                             codes, scales, tokens)
+        if r >= 0:
+            return codes, scales, tokens, r
+        _refused(ctx, r)
     _need(h, torch.float32, "h")
     if W_h.dtype == torch.bfloat16:
         wdt = SPH_DTYPE_BF16
@@ -452,6 +512,12 @@ def sph_verify_draft(ctx, target_logits, sessions: int, k: int, draft_tokens,
                      *, keep_ids=None, draft_probs=None, temperature=1.0,
                      seed=0, offset=0, n_accepted=None, next_token=None):
     """Speculative verification.  Returns (n_accepted, next_token)."""
+    if n_accepted is not None and next_token is not None:
+        r = _fast.verify_draft(_word(ctx), target_logits, sessions, k, draft_tokens, keep_ids,
+                               draft_probs, temperature, seed, offset, n_accepted, next_token)
+        if r >= 0:
+            return n_accepted, next_token
+        _refused(ctx, r)
     _need(target_logits, torch.float32, "target_logits")
     _need(draft_tokens, torch.int32, "draft_tokens")
     _need(draft_probs, torch.float32, "draft_probs")
@@ -487,7 +553,7 @@ class Context:
         self.handle = sph_create(self.device, self._stream)
 
     def _follow_stream(self):
-        s = torch.cuda.current_stream(self.device).cuda_stream
+        s = _raw_stream(self.device)
         if s != self._stream:
             sph_set_stream(self.handle, s)
             self._stream = s
