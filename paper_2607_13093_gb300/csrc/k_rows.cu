@@ -906,6 +906,22 @@ cudaError_t launch_sample_rows(const ZSource& zs, int rows, int n, const float2*
                           offset, tokens, st);
 }
 
+cudaError_t launch_sample_made_stats(const ZSource& zs, int rows, int n, const float2* stats,
+                                     int nseg, float2* cstats, const int32_t* ids,
+                                     float inv_tau, uint64_t seed, uint64_t offset,
+                                     int sm_count, int32_t* tokens, cudaStream_t st,
+                                     int greedy) {
+  if (greedy)   // the segment maxima are all greedy decoding needs
+    return launch_sample_segments(zs, rows, n, stats, nseg, nullptr, ids, inv_tau, seed, offset,
+                                  tokens, st, 1);
+  if (chunk_count(nseg) <= kMaxFusedChunks)
+    return launch_sample_rows(zs, rows, n, stats, nseg, ids, inv_tau, seed, offset, tokens, st);
+  cudaError_t e = launch_chunk_stats(stats, rows, nseg, inv_tau, cstats, sm_count, st);
+  if (e != cudaSuccess) return e;
+  return launch_sample_segments(zs, rows, n, stats, nseg, cstats, ids, inv_tau, seed, offset,
+                                tokens, st);
+}
+
 // Scratch: stats [R][nseg] float2 | chunk stats [R][nchunk] float2 | rowMS
 // [R] float2 | acc, xis [S*k] int32 | residual segment weights [S][nseg] |
 // residual chunk weights [S][nchunk], with R = S * (k + 1).

@@ -2002,16 +2002,8 @@ cudaError_t launch_sample_from_stats(const ZSource& zs, int rows, int n, const T
     return launch_sample_segments(zs, rows, n, sst, seg_count(n), cstats, ids, inv_tau, seed,
                                   offset, tokens, st, greedy);
   }
-  const int nseg = pl.nseg;
-  if (greedy)   // the segment maxima are all greedy decoding needs
-    return launch_sample_segments(zs, rows, n, stats, nseg, nullptr, ids, inv_tau, seed, offset,
-                                  tokens, st, 1);
-  if (chunk_count(nseg) <= 4096)
-    return launch_sample_rows(zs, rows, n, stats, nseg, ids, inv_tau, seed, offset, tokens, st);
-  cudaError_t e = launch_chunk_stats(stats, rows, nseg, inv_tau, cstats, sm_count, st);
-  if (e != cudaSuccess) return e;
-  return launch_sample_segments(zs, rows, n, stats, nseg, cstats, ids, inv_tau, seed, offset,
-                                tokens, st);
+  return launch_sample_made_stats(zs, rows, n, stats, pl.nseg, cstats, ids, inv_tau, seed, offset,
+                                  sm_count, tokens, st, greedy);
 }
 
 }  // namespace sph

@@ -15,6 +15,11 @@ namespace sph {
 thread_local long long launch_count = 0;
 }
 
+namespace {
+constexpr int64_t kTcMinRows = 4;              // SPH_OPT_TC_MIN_ROWS
+constexpr long long kFinishWait = 1ll << 15;   // SPH_OPT_TC_FINISH_WAIT
+}
+
 struct ProfPair {
   int cls;
   cudaEvent_t start, stop;
@@ -28,14 +33,14 @@ struct sph_ctx {
   void* scratch = nullptr;          // arena for per-call temporaries
   size_t scratch_cap = 0;
   unsigned* status = nullptr;       // device error word (sph::ERR_* bits)
-  int64_t tc_min_rows = 4;          // SPH_OPT_TC_MIN_ROWS
+  int64_t tc_min_rows = kTcMinRows; // SPH_OPT_TC_MIN_ROWS
   long long spin_limit = 1ll << 34; // SPH_OPT_SPIN_LIMIT
   int tc_schedule = 0;              // SPH_OPT_TC_SCHEDULE
   int tc_stages = 0;                // SPH_OPT_TC_STAGES
   int tc_block_k = 0;               // SPH_OPT_TC_BLOCK_K
   int tc_max_bn = 0;                // SPH_OPT_TC_MAX_BN
   int tc_tile_m = 0;                // SPH_OPT_TC_TILE_M
-  long long tc_finish_wait = 1ll << 15;   // SPH_OPT_TC_FINISH_WAIT
+  long long tc_finish_wait = kFinishWait;   // SPH_OPT_TC_FINISH_WAIT
   int sampler = 0;                  // SPH_OPT_SAMPLER
   int check_ids = 0;                // SPH_OPT_CHECK_IDS
   int split_quantize = 0;           // SPH_OPT_SPLIT_QUANTIZE
@@ -151,6 +156,43 @@ bool use_tc(const sph_ctx* ctx, int64_t rows, int w_dtype) {
 int pair_mode(const sph_ctx* ctx) {
   if (ctx->pair_units < 1 || ctx->tc_pair == 2) return 0;
   return ctx->tc_pair == 1 ? 2 : 1;
+}
+
+// The tensor-core kernel's options all at their defaults: an explicit
+// crossover, schedule, tile, pair mode or z choice asks for the general
+// kernel, whose choices they are.
+bool default_tc_options(const sph_ctx* ctx) {
+  return ctx->tc_min_rows == kTcMinRows && ctx->tc_schedule == 0 && ctx->tc_stages == 0 &&
+         ctx->tc_block_k == 0 && ctx->tc_max_bn == 0 && ctx->tc_tile_m == 0 &&
+         ctx->tc_finish_wait == kFinishWait && ctx->tc_pair == 0 && ctx->endpoint_rm == 0 &&
+         ctx->endpoint_z != 2;
+}
+// Whether an endpoint contraction takes the few-row kernel, and its plan on
+// sm_count SMs: 4..32 rows over at most 512 columns, where the general
+// kernel would take whole tiles as well.  Endpoint call with its draw,
+// general against few-row kernel, us: 32 rows x 12000 ids x 256 13.3 / 9.9,
+// x 60000 x 96 25.4 / 16.9, x 256000 x 512 83.4 / 77.7; 12 rows x 44999 x 512
+// 27.1 / 21.1; 4 rows x 700 x 48 11.0 / 7.1.  Past 512 columns the copies'
+// arrivals weigh more than the launch and the set-up saved (32 rows x 60000 x
+// 1024 43.9 / 51.3, 24 x 152064 x 1024 79.8 / 89.7).  Over whole tiles both
+// kernels add in the same order, so z has the same bits; where the general
+// kernel would split a tile's columns over CTAs its shorter chains round a
+// little less, and it stays.
+bool few_shape(const sph_ctx* ctx, int64_t rows, int64_t n, int64_t K, bool gather, int sm_count,
+               sph::FewPlan* pl) {
+  if (rows < ctx->tc_min_rows || rows > sph::kFewMaxRows || K > sph::kFewMaxK ||
+      !default_tc_options(ctx))
+    return false;
+  if (!sph::tc_plan((int)rows, (int)n, (int)K, 0, sm_count, 1, 0, 0, 0, gather, 0, 0, 0,
+                    pair_mode(ctx), ctx->pair_units, 0)
+           .whole_tiles)
+    return false;
+  *pl = sph::few_plan((int)rows, (int)n, (int)K, sm_count);
+  return pl->ok;
+}
+bool few_route(const sph_ctx* ctx, const sph::GatherGemm& g, int sm_count, sph::FewPlan* pl) {
+  return sph::few_operands(g) &&
+         few_shape(ctx, g.rows, g.n, g.K, g.ids != nullptr, sm_count, pl);
 }
 
 size_t tc_bytes(const sph_ctx* ctx, int64_t rows, int64_t n, int64_t K, int act_bf16,
@@ -359,7 +401,9 @@ sph_status endpoint_draw(sph_ctx* ctx, sph::GatherGemm& gg, Carve& c, float temp
   // lane (measured, steps of 1024 x 256000 ids x d_l 512: 3.18 vs 3.43 ms;
   // 256 x 152064 x 1024: 0.87 vs 0.90 ms; 256 x 256000 x 512: 0.88 vs
   // 1.00 ms), not with ids as M (32 x 12000 x 256: 55 vs 49 us)
-  const bool tc = use_tc(ctx, rows, sph::W_BF16);
+  sph::FewPlan few{};
+  const bool is_few = few_route(ctx, gg, ctx->sm_count, &few);
+  const bool tc = !is_few && use_tc(ctx, rows, sph::W_BF16);
   bool z_free = tc && !gumbel && !z_out && ctx->endpoint_z != 1;
   auto plan_of = [&](bool zf) {
     return sph::tc_plan(rows, n_keep, gg.K, 0, ctx->sm_count, zf ? 2 : 1, ctx->tc_schedule,
@@ -415,6 +459,18 @@ sph_status endpoint_draw(sph_ctx* ctx, sph::GatherGemm& gg, Carve& c, float temp
   if (!c.fits())
     return fail(ctx, SPH_ERR_UNSUPPORTED, "internal: scratch plan of %zu bytes exceeds the arena of %zu",
                 c.off, ctx->scratch_cap);
+  if (is_few) {
+    st = launch_status(ctx, traced(ctx, SPH_PROF_LOCAL_GEMM, [&] {
+                         return sph::launch_few(gg, few, stats, ctx->spin_limit, ctx->stream);
+                       }), "few-row launch");
+    if (st || fuse_only) return st;
+    if (gumbel) return draw_gumbel();
+    return launch_status(ctx, traced(ctx, SPH_PROF_SAMPLE, [&] {
+                           return sph::launch_sample_made_stats(
+                               zs, rows, n_keep, stats, few.nseg, cstats, keep_ids, gg.inv_tau,
+                               seed, offset, ctx->sm_count, tokens, ctx->stream, greedy);
+                         }), "sample launch");
+  }
   st = launch_status(ctx, traced(ctx, SPH_PROF_LOCAL_GEMM, [&] {
                        return sph::launch_gemv(gg, ctx->sm_count, ctx->stream);
                      }), "gemv launch");
@@ -497,6 +553,21 @@ sph_status sph_plan_query(sph_ctx* ctx, int call, int64_t rows, int64_t n_keep, 
     return fail(ctx, SPH_ERR_INVALID_ARG, "sph_plan_query: bad arguments");
   *out = sph_plan{};
   const int wdt = w_dtype == SPH_DTYPE_BF16 ? sph::W_BF16 : sph::W_FP8;
+  sph::FewPlan few{};
+  if (call == 1 && few_shape(ctx, rows, n_keep, K, gather != 0, ctx->sm_count, &few)) {
+    out->tensor_core = 1;
+    out->row_blocks = 1;
+    out->block_rows = rows <= 16 ? 16 : 32;
+    out->tile_ids = few.pitch;
+    out->tiles = few.tiles;
+    out->k_blocks = few.KB;
+    out->stages = few.stages;
+    out->grid = few.grid;
+    out->whole_tiles = 1;
+    out->planes = 2;
+    out->epilogue_stats = 1;
+    return SPH_OK;
+  }
   if (!use_tc(ctx, rows, wdt)) {
     out->gemv_rows = sph::gemv_rows_per_launch((int)rows, (int)K);
     return SPH_OK;
@@ -1154,7 +1225,11 @@ sph_status sph_split_step(sph_ctx* ctx, const float* h, int64_t rows, int64_t ld
     gg.Y = Z + j0; gg.ldy = n_keep;
     gg.status = ctx->status; gg.finish_wait = ctx->tc_finish_wait;
     gg.inv_tau = inv_tau; gg.no_stats = true;
-    if (use_tc(ctx, rows, sph::W_BF16)) {
+    sph::FewPlan few{};
+    if (few_route(ctx, gg, sm_end, &few)) {
+      st = launch_status(ctx, sph::launch_few(gg, few, nullptr, ctx->spin_limit, es),
+                         "few-row launch");
+    } else if (use_tc(ctx, rows, sph::W_BF16)) {
       const sph::TcPlan pl = sph::tc_plan((int)rows, (int)n_q, (int)d_l, 0, sm_end, 1,
                                           ctx->tc_schedule, ctx->tc_stages, ctx->tc_block_k,
                                           keep_ids != nullptr, 0, ctx->tc_max_bn, ctx->tc_tile_m);

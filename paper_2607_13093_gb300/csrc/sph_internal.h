@@ -164,6 +164,29 @@ int tc_pair_max_units(int device);
 // plan.scratch_bytes bytes.  bf16 weights only.
 cudaError_t launch_tc(const GatherGemm& g, const TcPlan& plan, void* scratch,
                       long long spin_limit, cudaStream_t st);
+// Few-row endpoint contraction over a short hidden dimension (k_few.cu): one
+// CTA per SM takes tiles of at most 128 kept ids, the hidden states of all
+// rows stay in its shared memory.
+constexpr int kFewMaxRows = 32;
+constexpr int kFewMaxK = 512;
+struct FewPlan {
+  int pitch;       // kept ids of a tile: 32, 64, 96 or 128
+  int na, KB;      // 64-column atoms of a stage, stages of a tile
+  int tiles;
+  int grid;        // persistent CTAs, one per SM at most
+  int stages, lag; // ring depth; stages copied before a tile's epilogue waits
+  int nseg;        // 32-id segments per row of the statistics
+  size_t smem_bytes;
+  bool ok;
+};
+FewPlan few_plan(int rows, int n, int K, int sm_count);
+// What the kernel takes: EPI_ENDPOINT or EPI_FUSED, bf16 weights with 16-byte
+// aligned rows.
+bool few_operands(const GatherGemm& g);
+// seg_stats receives, unless g.no_stats, the statistics [rows][plan.nseg].
+cudaError_t launch_few(const GatherGemm& g, const FewPlan& plan, float2* seg_stats,
+                       long long spin_limit, cudaStream_t st);
+
 // Where a draw finds the fused logits of the ids it visits (the 32 ids of
 // the segment it lands in): stored in Z (fp32 [rows, n]), or, with Z null,
 // recomputed for just those ids from the endpoint call's own inputs (Eq. 13),
@@ -241,6 +264,14 @@ inline cudaError_t launch_sample_segments(const float* Z, int rows, int n,
   return launch_sample_segments(zs, rows, n, stats, nseg, cstats, ids, inv_tau, seed, offset,
                                 tokens, st, greedy);
 }
+// One draw per row (greedy: the argmax) from segment statistics a
+// contraction's epilogue made: the fused sampler, or past its 4096 chunks a
+// chunk-statistics pass into cstats and the segment sampler.
+cudaError_t launch_sample_made_stats(const ZSource& zs, int rows, int n, const float2* stats,
+                                     int nseg, float2* cstats, const int32_t* ids,
+                                     float inv_tau, uint64_t seed, uint64_t offset,
+                                     int sm_count, int32_t* tokens, cudaStream_t st,
+                                     int greedy);
 int sample_max_n();
 int verify_max_k();
 

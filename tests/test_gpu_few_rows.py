@@ -1,0 +1,105 @@
+"""The endpoint's few-row kernel (4..32 rows over at most 512 columns) at the
+edges of its tiles, turns, rows and columns, against the oracle and, bit for
+bit, against the general tensor-core kernel it takes over from (both add in
+the same order over whole tiles).  Needs a GPU (marked gpu)."""
+import pytest
+import torch
+
+from paper_2607_13093_gb300 import workloads as wl
+from _parity import check_endpoint
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2607_13093_gb300 import build_lib
+    build_lib.build()
+    from paper_2607_13093_gb300 import sph
+    c = sph.Context(0)
+    yield c
+    c.close()
+
+
+def general(ctx, f):
+    """f() on the general kernel (an explicit option asks for it)."""
+    from paper_2607_13093_gb300 import sph
+    ctx.set_option(sph.SPH_OPT_TC_FINISH_WAIT, (1 << 15) - 1)
+    try:
+        return f()
+    finally:
+        ctx.set_option(sph.SPH_OPT_TC_FINISH_WAIT, 1 << 15)
+
+
+# rows (4, both sides of 16, 32), kept ids (segments, tiles and SM turns: one
+# turn of 152 tiles ends at 19456 ids), columns (atoms of 64, stages of 128)
+CASES = [(4, 1, 48), (5, 31, 8), (16, 33, 64), (17, 128, 65), (32, 129, 128), (31, 700, 96),
+         (8, 4864, 130), (32, 4865, 200), (12, 19456, 63), (9, 19457, 16), (32, 60000, 96),
+         (6, 40001, 256), (16, 30011, 512), (32, 12000, 512)]
+
+
+@pytest.mark.parametrize("rows,n,K", CASES)
+@pytest.mark.parametrize("payload", [True, False])
+def test_few_rows(ctx, rows, n, K, payload):
+    V = max(n + n // 3, 64)
+    w = wl.make_workload(V=V, d=K + 24, d_l=K, rows=rows, n_keep=n, tau=0.8, seed=900 + n + K,
+                         device=DEV, run_lo=1 if n < 64 else 16, run_hi=3 if n < 64 else 256)
+    if K % 8:        # weight rows of a padded stride, junk past the columns
+        Wp = torch.full((V, (K + 7) // 8 * 8), float("nan"), dtype=torch.bfloat16, device=DEV)
+        Wp[:, :K] = w.W_l
+        w.W_l = Wp[:, :K]
+    assert ctx.plan(1, rows, n, K)["block_rows"] in (16, 32)
+    pc, ps = wl.make_payload(rows, n, seed=3, device=DEV) if payload else (None, None)
+
+    def run():
+        z = torch.full((rows, n), 7.0, device=DEV)
+        t = ctx.fuse_sample(pc, ps, w.h_local, w.W_l, keep_ids=w.keep_ids, temperature=w.tau,
+                            seed=w.seed, offset=5, fused_logits_out=z)
+        g = ctx.fuse_sample(pc, ps, w.h_local, w.W_l, keep_ids=w.keep_ids, temperature=0.0)
+        y = torch.full((rows, n), 7.0, device=DEV)
+        ctx.fuse_sample(pc, ps, w.h_local, w.W_l, keep_ids=w.keep_ids, draw=False,
+                        fused_logits_out=y)
+        ctx.sync()
+        return z, t, g, y
+
+    a, b = run(), general(ctx, run)
+    for x, y in zip(a, b):
+        assert torch.equal(x, y)
+    assert torch.equal(a[0], a[3])
+    if payload and K % 8 == 0:
+        check_endpoint(ctx, w, pc.cpu(), ps.cpu(), unstored=False)
+
+
+@pytest.mark.parametrize("rows,n,chunk", [(19, 11987, 0), (4, 3001, 0), (32, 30000, 10000)])
+def test_few_rows_one_call(ctx, rows, n, chunk):
+    # the fused quantizing epilogue, and the endpoint of a block-streamed
+    # payload, against the general kernel; hidden states in rows that are not
+    # 16-byte aligned
+    w = wl.make_workload(V=n + 999, d=640, d_l=256, rows=rows, n_keep=n, seed=31, device=DEV)
+    hp = torch.zeros(rows, 641, device=DEV)
+    for h in (w.h, hp[:, 1:].copy_(w.h)):
+        def run():
+            z = torch.empty(rows, n, device=DEV)
+            c, s, t, _ = ctx.split_step(h, w.d_l, w.W_h, w.W_l, keep_ids=w.keep_ids,
+                                        temperature=0.9, seed=4, chunk=chunk, fused_logits_out=z)
+            ctx.sync()
+            return c, s, t, z
+        for x, y in zip(run(), general(ctx, run)):
+            assert torch.equal(x, y)
+
+
+def test_few_rows_wait_timeout_is_reported_and_context_recovers(ctx):
+    from paper_2607_13093_gb300 import sph
+    w = wl.make_workload(V=60000, d=320, d_l=256, rows=20, n_keep=30000, device=DEV, seed=93)
+    pc, ps = wl.make_payload(w.rows, w.n_keep, seed=3)
+    ctx.set_option(sph.SPH_OPT_SPIN_LIMIT, 1)
+    try:
+        ctx.fuse_sample(pc.to(DEV), ps.to(DEV), w.h_local, w.W_l, keep_ids=w.keep_ids)
+        with pytest.raises(sph.SphError) as err:
+            ctx.sync()
+        assert err.value.status == 4, str(err.value)
+    finally:
+        ctx.set_option(sph.SPH_OPT_SPIN_LIMIT, 1 << 34)
+    ctx.sync()
+    check_endpoint(ctx, w, pc, ps, unstored=False)
