@@ -19,7 +19,7 @@
 //       then lo, in the order of the general kernel, so z has the same bits.
 //
 // Warps 0-7 copy and run the epilogue; warp 8 owns TMEM and issues the MMAs
-// (one thread).  The copies of the next tiles are in flight while a tile's
+// (one elected lane).  The copies of the next tiles are in flight while a tile's
 // epilogue runs.  Every wait is bounded; a wait that gives up sets the
 // context's error word, and the CTA winds down after its copies and MMAs have
 // landed.
@@ -170,51 +170,55 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
     s_abort = 1;
   };
 
+  auto warp_wait = [&](uint64_t* bar, uint32_t parity) {
+    const bool ok = __all_sync(0xFFFFFFFFu, !s_abort && ptx::mbar_wait(bar, parity, limit));
+    if (!ok && lane == 0 && !s_abort) give_up();
+    return ok;
+  };
+
   if (warp == kWorkWarps) {
     // ---------------------------------------------------------- MMA issuer
+    // (the whole warp runs the loop, one elected lane issues: see the PTX
+    // wrappers)
     ptx::griddep_launch_dependents();
-    if (lane == 0) {
-      constexpr uint32_t idesc = ptx::idesc_bf16_f32(kTileIds, NR);
-      int stage = 0;
-      uint32_t phase = 0;
-      bool stop = !ptx::mbar_wait(&s_hready, 0, limit);
-      if (stop && !s_abort) give_up();
-      for (int x = 0; x < my_tiles && !stop; ++x) {
-        const int acc = x & 1;
-        // (the accumulator's previous tile, x - 2, has been read)
-        if (x >= 2 && (s_abort || !ptx::mbar_wait(&s_tempty[acc], (uint32_t)((x >> 1) - 1) & 1u,
-                                                  limit))) {
-          if (!s_abort) give_up();
+    constexpr uint32_t idesc = ptx::idesc_bf16_f32(kTileIds, NR);
+    int stage = 0;
+    uint32_t phase = 0;
+    bool stop = !warp_wait(&s_hready, 0);
+    for (int x = 0; x < my_tiles && !stop; ++x) {
+      const int acc = x & 1;
+      // (the accumulator's previous tile, x - 2, has been read)
+      if (x >= 2 && !warp_wait(&s_tempty[acc], (uint32_t)((x >> 1) - 1) & 1u)) break;
+      const uint32_t d = tmem + (uint32_t)(acc * NR);
+      uint32_t hd = ptx::sdesc_k128(base);
+      uint32_t accum = 0;                      // the tile's first MMA overwrites
+      for (int kb = 0; kb < KB; ++kb) {
+        if (!warp_wait(&s_full[stage], phase)) {
+          stop = true;
           break;
         }
-        for (int kb = 0; kb < KB; ++kb) {
-          if (s_abort || !ptx::mbar_wait(&s_full[stage], phase, limit)) {
-            if (!s_abort) give_up();
-            stop = true;
-            break;
-          }
-          fence_proxy_async();
-          ptx::tc_fence_after();
-          const uint32_t d = tmem + (uint32_t)(acc * NR);
-          for (int at = 0; at < na; ++at) {
-            const uint32_t a0 = a_base + (uint32_t)stage * stage_bytes + (uint32_t)at * a_atom;
-            const uint32_t b0 = base + (uint32_t)(kb * na + at) * 2 * kHAtom;
+        fence_proxy_async();
+        ptx::tc_fence_after();
+        uint32_t wd = ptx::sdesc_k128(a_base + (uint32_t)stage * stage_bytes);
+        for (int at = 0; at < na; ++at) {
 #pragma unroll
-            for (int hl = 0; hl < 2; ++hl)
+          for (int hl = 0; hl < 2; ++hl)
 #pragma unroll
-              for (int kk = 0; kk < kAtomCols / 16; ++kk)
-                ptx::umma_f16(d, ptx::sdesc_k128(a0 + kk * 32),
-                              ptx::sdesc_k128(b0 + hl * kHAtom + kk * 32), idesc,
-                              (kb | at | hl | kk) ? 1u : 0u);
-          }
-          ptx::umma_commit(&s_empty[stage]);
-          if (++stage == S) { stage = 0; phase ^= 1; }
+            for (int kk = 0; kk < kAtomCols / 16; ++kk) {
+              ptx::umma_f16(d, wd + (uint32_t)(kk * 32 >> 4),
+                            hd + (uint32_t)((hl * kHAtom + kk * 32) >> 4), idesc, accum);
+              accum = 1;
+            }
+          wd += a_atom >> 4;
+          hd += 2 * kHAtom >> 4;
         }
-        if (!stop) ptx::umma_commit(&s_tfull[acc]);
+        ptx::umma_commit(&s_empty[stage]);
+        if (++stage == S) { stage = 0; phase ^= 1; }
       }
-      ptx::umma_commit(&s_drain);
-      ptx::mbar_wait(&s_drain, 0, kDrainLimit);
+      if (!stop) ptx::umma_commit(&s_tfull[acc]);
     }
+    ptx::umma_commit(&s_drain);
+    ptx::mbar_wait(&s_drain, 0, kDrainLimit);
     __syncwarp();
   } else {
     // ---------------------------------------------------- copy and epilogue
@@ -335,11 +339,6 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
     if (lane == 0) ptx::mbar_arrive(&s_hready);
     ptx::named_bar_sync(1, kWorkers);          // (s_rq)
 
-    auto warp_wait = [&](uint64_t* bar, uint32_t parity) {
-      const bool ok = __all_sync(0xFFFFFFFFu, !s_abort && ptx::mbar_wait(bar, parity, limit));
-      if (!ok && lane == 0 && !s_abort) give_up();
-      return ok;
-    };
     auto epilogue = [&](int x, int tile) -> bool {
       const int acc = x & 1;
       if (!warp_wait(&s_tfull[acc], (uint32_t)(x >> 1) & 1u)) return false;

@@ -38,7 +38,7 @@
 // either way, so results are deterministic.
 //
 // Warp roles: warp 0 issues the TMA copies, warp 1 owns TMEM and issues
-// tcgen05.mma (one thread), warps 2-9 drain the accumulator (double-buffered,
+// tcgen05.mma (one elected lane), warps 2-9 drain the accumulator (double-buffered,
 // or single for 256-row tiles over more than 128 rows) with tcgen05.ld and
 // run the fused epilogue -- two warps per TMEM lane quadrant, so that the
 // epilogue's dependent shuffle / exp chains of one warp overlap with the
@@ -549,7 +549,8 @@ tc_kernel(const __grid_constant__ WMaps wm,
   constexpr int kAtomE = FP8 ? kAtomE8 : kAtomK;   // elements per 128-byte atom
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = ptx::smem_u32(smem_raw);
-  uint8_t* base = smem_raw + (((raw_addr + 1023) & ~1023u) - raw_addr);
+  const uint32_t base_addr = (raw_addr + 1023) & ~1023u;
+  uint8_t* base = smem_raw + (base_addr - raw_addr);
   constexpr int kHalves = TM / 128;     // M = 128 halves of a tile
   constexpr int kGroups = TM / 32;      // 32-row lane groups of a tile
   constexpr int kTileStride = PAIR ? 256 : TM;      // ids between tiles
@@ -847,83 +848,80 @@ tc_kernel(const __grid_constant__ WMaps wm,
     // pair, odd CTA: the even CTA issues the MMAs for both
   } else if (warp == 1) {
     // ---------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      Segments sg{it0, it1, p.KB};
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t tph[2] = {0, 0};
-      int si = 0, tile, kb0, kb1;
-      constexpr int kMmaM = PAIR ? 2 * kTileM : kTileM;
-      const uint32_t idesc =
-          FP8 ? ptx::idesc_e4m3_f32(kMmaM, BN)
-              : ptx::idesc_bf16_f32(kMmaM, rm ? kTileStride : BN);   // (rows as M: N = ids)
-      auto wait_x = [&](uint64_t* bar, uint32_t parity) {
-        return ptx::mbar_wait(bar, parity, limit);
-      };
-      // accumulator `acc`, tile half hf: TMEM columns (acc * kHalves + hf) * BN
-      bool stop = false;
-      while (!stop && sg.next(tile, kb0, kb1)) {
-        const int acc = p.single_acc ? 0 : (si & 1);
-        if (*s_abort || !wait_x(&tempty[acc], tph[acc] ^ 1)) {
-          if (!*s_abort) give_up();
+    // (the whole warp runs the loop, one elected lane issues: see the PTX
+    // wrappers)
+    Segments sg{it0, it1, p.KB};
+    int stage = 0;
+    uint32_t phase = 0;
+    uint32_t tph[2] = {0, 0};
+    int si = 0, tile, kb0, kb1;
+    constexpr int kMmaM = PAIR ? 2 * kTileM : kTileM;
+    const uint32_t idesc =
+        FP8 ? ptx::idesc_e4m3_f32(kMmaM, BN)
+            : ptx::idesc_bf16_f32(kMmaM, rm ? kTileStride : BN);   // (rows as M: N = ids)
+    auto warp_wait = [&](uint64_t* bar, uint32_t parity) {
+      const bool ok = __all_sync(0xFFFFFFFFu, !*s_abort && ptx::mbar_wait(bar, parity, limit));
+      if (!ok && lane == 0 && !*s_abort) give_up();
+      return ok;
+    };
+    // accumulator `acc`, tile half hf: TMEM columns (acc * kHalves + hf) * BN
+    bool stop = false;
+    while (!stop && sg.next(tile, kb0, kb1)) {
+      const int acc = p.single_acc ? 0 : (si & 1);
+      if (!warp_wait(&tempty[acc], tph[acc] ^ 1)) break;
+      tph[acc] ^= 1;
+      ptx::tc_fence_after();
+      const uint32_t d = tmem_base + (uint32_t)(acc * kHalves * BN);
+      uint32_t accum = 0;                      // the tile's first MMA of each half overwrites
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!warp_wait(&full[stage], phase)) {
+          stop = true;
           break;
         }
-        tph[acc] ^= 1;
         ptx::tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(acc * kHalves * BN);
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (*s_abort || !wait_x(&full[stage], phase)) {
-            if (!*s_abort) give_up();
-            stop = true;
-            break;
-          }
-          ptx::tc_fence_after();
-          const uint32_t a0 = ptx::smem_u32(base + (size_t)stage * stage_bytes);
-          const uint32_t b0 = a0 + a_bytes;
-          for (int at = 0; at < NA; ++at) {
+        const uint32_t a0 = base_addr + (uint32_t)(stage * stage_bytes);
+        uint32_t wd0 = ptx::sdesc_k128(a0);
+        uint32_t hd0 = ptx::sdesc_k128(a0 + (uint32_t)a_bytes);
+        const uint32_t h_step = (uint32_t)(NA * BNc * 128) >> 4;    // one h plane
+        for (int at = 0; at < NA; ++at) {
 #pragma unroll
-            for (int h = 0; h < HILO; ++h) {
+          for (int h = 0; h < HILO; ++h) {
 #pragma unroll
-              for (int kk = 0; kk < kAtomK / 16; ++kk) {
+            for (int kk = 0; kk < kAtomK / 16; ++kk) {
+              // 32 bytes of K per MMA: 16 bf16 or 32 e4m3 elements
+              const uint32_t hd = hd0 + (uint32_t)h * h_step + (uint32_t)(kk * 32 >> 4);
 #pragma unroll
-                for (int hf = 0; hf < kHalves; ++hf)
-                {
-                  // 32 bytes of K per MMA: 16 bf16 or 32 e4m3 elements
-                  const uint64_t wd =
-                      ptx::sdesc_k128(a0 + at * atom_bytes + hf * kAtomBytes + kk * 32);
-                  const uint64_t hd = ptx::sdesc_k128(b0 + (h * NA + at) * BNc * 128 + kk * 32);
-                  const uint64_t ad = rm ? hd : wd, bd = rm ? wd : hd;
-                  const uint32_t accum = (kb != kb0 || at != 0 || h != 0 || kk != 0) ? 1u : 0u;
-                  if constexpr (PAIR && FP8)
-                    ptx::umma_f8_pair(d, ad, bd, idesc, accum);
-                  else if constexpr (PAIR)
-                    ptx::umma_f16_pair(d, ad, bd, idesc, accum);
-                  else if constexpr (FP8)
-                    ptx::umma_f8(d + (uint32_t)(hf * BN), ad, bd, idesc, accum);
-                  else
-                    ptx::umma_f16(d + (uint32_t)(hf * BN), ad, bd, idesc, accum);
-                }
+              for (int hf = 0; hf < kHalves; ++hf) {
+                const uint32_t wd = wd0 + (uint32_t)((hf * kAtomBytes + kk * 32) >> 4);
+                const uint32_t ad = rm ? hd : wd, bd = rm ? wd : hd;
+                if constexpr (PAIR && FP8)
+                  ptx::umma_f8_pair(d, ad, bd, idesc, accum);
+                else if constexpr (PAIR)
+                  ptx::umma_f16_pair(d, ad, bd, idesc, accum);
+                else if constexpr (FP8)
+                  ptx::umma_f8(d + (uint32_t)(hf * BN), ad, bd, idesc, accum);
+                else
+                  ptx::umma_f16(d + (uint32_t)(hf * BN), ad, bd, idesc, accum);
               }
+              accum = 1;
             }
           }
-          if constexpr (PAIR) ptx::umma_commit_pair(&empty[stage]);
-          else ptx::umma_commit(&empty[stage]);
-          if (++stage == S) { stage = 0; phase ^= 1; }
+          wd0 += (uint32_t)atom_bytes >> 4;
+          hd0 += (uint32_t)(BNc * 128) >> 4;
         }
-        if (stop) break;
-        if constexpr (PAIR) ptx::umma_commit_pair(&tfull[acc]);
-        else ptx::umma_commit(&tfull[acc]);
-        ++si;
+        if constexpr (PAIR) ptx::umma_commit_pair(&empty[stage]);
+        else ptx::umma_commit(&empty[stage]);
+        if (++stage == S) { stage = 0; phase ^= 1; }
       }
-      // all issued MMAs complete before TMEM is released
-      if constexpr (PAIR) {
-        ptx::umma_commit_pair(drain);
-        ptx::mbar_wait(drain, 0, kDrainLimit);
-      } else {
-        ptx::umma_commit(drain);
-        ptx::mbar_wait(drain, 0, kDrainLimit);
-      }
+      if (stop) break;
+      if constexpr (PAIR) ptx::umma_commit_pair(&tfull[acc]);
+      else ptx::umma_commit(&tfull[acc]);
+      ++si;
     }
+    // all issued MMAs complete before TMEM is released
+    if constexpr (PAIR) ptx::umma_commit_pair(drain);
+    else ptx::umma_commit(drain);
+    ptx::mbar_wait(drain, 0, kDrainLimit);
   } else if (warp < 2 + kEpiWarps) {
     // ------------------------------------------------------------ epilogue
     // A warp may only read the TMEM lanes of its quadrant (warp index mod

@@ -103,18 +103,26 @@ __device__ __forceinline__ void tc_fence_after() {
 }
 
 // ---- tcgen05.mma ------------------------------------------------------------
+// Whole warps run the MMA loops and one elected lane of theirs issues: the
+// loop's counters, addresses and descriptors are then warp-uniform and stay
+// in the uniform registers that the instruction takes its operands from (a
+// loop run by a single lane moves each one there first: 75-100 cycles an MMA,
+// longer than a short MMA itself; steps before and after: 32 rows x 12000 ids
+// 44.4 -> 43.5 us, 32 x 60000 118.2 -> 114.9, the drafted 320 x 51302 293.9 ->
+// 287.2, 1024 x 256000 3367 -> 3317).  elect.sync elects the same lane every
+// time, so commits cover the MMAs.
+//
 // Shared-memory matrix descriptor: K-major operand stored as 8-row groups of
 // 128-byte rows with the 128-byte swizzle (the layout TMA's SWIZZLE_128B
-// produces), groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t sdesc_k128(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);      // start address
-  d |= (uint64_t)1 << 16;                        // leading offset (unused)
-  d |= (uint64_t)(1024 >> 4) << 32;              // stride offset: 8 rows
-  d |= (uint64_t)1 << 46;                        // descriptor version
-  d |= (uint64_t)2 << 61;                        // 128-byte swizzle
-  return d;
+// produces), groups 1024 bytes apart.  sdesc_k128 is the low word (start
+// address; leading offset, unused); another operand piece at a 16-byte
+// multiple `off` further on is the word plus off >> 4.
+__device__ __forceinline__ uint32_t sdesc_k128(uint32_t saddr) {
+  return (saddr >> 4) | (1u << 16);
 }
+constexpr uint32_t kSdescHi = (1024u >> 4)       // stride offset: 8 rows
+                              | (1u << 14)       // descriptor version
+                              | (2u << 29);      // 128-byte swizzle
 // Instruction descriptor for kind::f16 with bf16 A/B, fp32 D, K-major A/B.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
@@ -126,30 +134,31 @@ __host__ __device__ constexpr uint32_t idesc_e4m3_f32(int M, int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 // tcgen05.mma kind::f8f6f4 (8-bit operands; 32 elements of K per MMA)
-__device__ __forceinline__ void umma_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+__device__ __forceinline__ void umma_f8(uint32_t d_tmem, uint32_t adesc, uint32_t bdesc,
                                         uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n elect.sync _|q, 0xFFFFFFFF;\n"
+      " setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+      " @q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a, b, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(adesc), "r"(bdesc), "r"(idesc), "r"(accumulate), "r"(kSdescHi)
       : "memory");
 }
 // tcgen05.mma kind::f16 (the operand types come from the instruction
 // descriptor: bf16 x bf16 here)
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc,
-                                          uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
+__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint32_t adesc, uint32_t bdesc,
+                                        uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n elect.sync _|q, 0xFFFFFFFF;\n"
+      " setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(adesc), "r"(bdesc), "r"(idesc), "r"(accumulate), "r"(kSdescHi)
       : "memory");
 }
-// Arrive on `bar` once all previously issued tcgen05.mma of this thread are
-// complete.
+// Arrive on `bar` once all MMAs the elected lane has issued are complete.
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+      "{\n .reg .pred q;\n elect.sync _|q, 0xFFFFFFFF;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(
           smem_u32(bar))
       : "memory");
 }
@@ -243,30 +252,32 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 // M = 256 over the pair: A rows 0-127 from this CTA's shared memory and rows
 // 128-255 from the peer's at the same offset; B columns 0 .. N/2-1 from this
 // CTA and N/2 .. N-1 from the peer; D (128 lanes x N columns) into each
-// CTA's tensor memory at the same address.  Issued by one thread of the
-// even CTA.
-__device__ __forceinline__ void umma_f16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                              uint32_t idesc, uint32_t accumulate) {
+// CTA's tensor memory at the same address.  Issued by the even CTA.
+__device__ __forceinline__ void umma_f16_pair(uint32_t d_tmem, uint32_t adesc, uint32_t bdesc,
+                                        uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n elect.sync _|q, 0xFFFFFFFF;\n"
+      " setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(adesc), "r"(bdesc), "r"(idesc), "r"(accumulate), "r"(kSdescHi)
       : "memory");
 }
-__device__ __forceinline__ void umma_f8_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                             uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_f8_pair(uint32_t d_tmem, uint32_t adesc, uint32_t bdesc,
+                                        uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n elect.sync _|q, 0xFFFFFFFF;\n"
+      " setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+      " @q tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], a, b, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(adesc), "r"(bdesc), "r"(idesc), "r"(accumulate), "r"(kSdescHi)
       : "memory");
 }
 // Arrive on the mbarrier at local offset `bar` in both CTAs of the pair once
-// this thread's earlier pair MMAs are complete.
+// the elected lane's earlier pair MMAs are complete.
 __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
   asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-      " [%0], %1;" ::"r"(smem_u32(bar)),
+      "{\n .reg .pred q;\n elect.sync _|q, 0xFFFFFFFF;\n"
+      " @q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster"
+      ".multicast::cluster.b64 [%0], %1;\n}\n" ::"r"(smem_u32(bar)),
       "h"((uint16_t)3)
       : "memory");
 }
