@@ -276,9 +276,10 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
         for (int q = 0; q < 16; ++q)
           pay_f[q] = __ldcg(p.yc + (int64_t)min(erow0 + q, p.R - 1) * p.n + j);
       } else if (p.codes) {
+        const int8_t* cp = p.codes + (int64_t)erow0 * p.n + j;
 #pragma unroll
-        for (int q = 0; q < 16; ++q)
-          pay_c[q] = __ldg(p.codes + (int64_t)min(erow0 + q, p.R - 1) * p.n + j);
+        for (int q = 0; q < 16; ++q, cp += p.n)
+          if (erow0 + q < p.R) pay_c[q] = __ldg(cp);
       }
     };
 #pragma unroll
@@ -353,6 +354,39 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
       const int j = tile * p.pitch + quad * 32 + lane;
       const bool vj = j < p.n;
       const int kr = (lane >> 1) & 15;         // the row this lane reduces
+      if constexpr (EPI == EPI_ENDPOINT) {
+        // all 32 ids exist (nearly always): no lane predicate and no address
+        // product per value (an epilogue's length is its instructions'
+        // latency)
+        if (__all_sync(0xFFFFFFFFu, vj)) {
+          const int nr = p.R - erow0;
+          if (p.codes) {
+#pragma unroll
+            for (int q = 0; q < 16; ++q)
+              z[q] = z[q] + (float)pay_c[q] * s_rq[min(erow0 + q, NR - 1)].s;
+          }
+          if (p.Z) {
+            float* zp = p.Z + (int64_t)erow0 * p.ldz + j;
+#pragma unroll
+            for (int q = 0; q < 16; ++q, zp += p.ldz)
+              if (q < nr) *zp = z[q];
+          }
+          load_payload(tile + (int)gridDim.x);
+          if (p.seg_stats) {
+            const float mk = warp_reduce_scatter16(z, MaxOp{}, lane);
+            float e[16];
+            const float l2t = p.inv_tau * kLog2eF;
+#pragma unroll
+            for (int q = 0; q < 16; ++q)
+              e[q] = ex2_approx((z[q] - __shfl_sync(0xFFFFFFFFu, mk, 2 * q)) * l2t);
+            const float sk = warp_reduce_scatter16(e, SumOp{}, lane);
+            if (!(lane & 1) && kr < nr)
+              p.seg_stats[(int64_t)(erow0 + kr) * p.nseg + ((tile * p.pitch) >> 5) + quad] =
+                  make_float2(mk, sk);
+          }
+          return true;
+        }
+      }
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
         const int r = min(erow0 + q, p.R - 1);

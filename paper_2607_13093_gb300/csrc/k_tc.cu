@@ -197,8 +197,15 @@ __device__ __forceinline__ void load_payload(const TcParams& p, int row0, int j,
     return;
   }
   const int8_t* col = p.codes + min(j, p.n - 1);
+  if (row0 + 16 <= p.R) {
+    col += (int64_t)row0 * p.n;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) pl.c[q] = (float)__ldg(col + (int64_t)min(row0 + q, p.R - 1) * p.n);
+    for (int q = 0; q < 16; ++q, col += p.n) pl.c[q] = (float)__ldg(col);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      pl.c[q] = (float)__ldg(col + (int64_t)min(row0 + q, p.R - 1) * p.n);
+  }
   pl.s = __ldg(p.row_scale + min(row0 + (lane & 15), p.R - 1));
 }
 // Warm L2 with the payload of rows row0..row0+nrows-1 at the 32 ids from j0
@@ -220,6 +227,13 @@ __device__ __forceinline__ void prefetch_payload(const TcParams& p, int row0, in
 
 // Epilogue of 16 accumulator columns (hidden-state rows row0..row0+15) for
 // this lane's vocabulary column j (endpoint: with the chunk's payload).
+// A warp runs it alone on its scheduler or with one other, so its length is
+// its instructions' latency: chunks whose rows and ids all exist (nearly all)
+// take a path without a predicate and an address product per value (a cloud
+// chunk of few rows 2800 cycles with them, 1100 without; with the split tiles'
+// partials fetched a chunk ahead the decode step went from 43.5 to 42.9 us,
+// 32 rows x 60000 ids 114.9 -> 110.7, 320 x 51302 287.2 -> 273.7, unsplit 147 x
+// 32000 x 4096 95.3 -> 91.5).
 template <int EPI>
 __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)[16],
                                              int row0, int j, bool vj, int id,
@@ -231,6 +245,29 @@ __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)
     // times the weight row's scale and (below) the h row's scale
     const float ws = (vj && p.w_scale) ? p.w_scale[id] : 1.0f;
     float m[16];
+    if (row0 + 16 <= p.R && __all_sync(0xFFFFFFFFu, vj)) {
+      float y[16];
+      if (p.h_scale) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) y[q] = (v[q] * __ldg(p.h_scale + row0 + q)) * ws + b;
+      } else {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) y[q] = v[q] * ws + b;
+      }
+      const int64_t o = (int64_t)row0 * p.n + j;
+      if (p.partial_out) {
+        float* up = p.partial_out + o;
+#pragma unroll
+        for (int q = 0; q < 16; ++q, up += p.n) *up = y[q];
+      }
+      float* yp = p.Y + o;
+#pragma unroll
+      for (int q = 0; q < 16; ++q, yp += p.n) {
+        const float yc = fminf(fmaxf(y[q], -p.clip), p.clip);
+        *yp = yc;
+        m[q] = fabsf(yc);
+      }
+    } else
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
       const int r = row0 + q;
@@ -249,6 +286,34 @@ __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)
       atomicMax(&p.rowmax[row0 + kr], __float_as_uint(mr));
   } else {
     float z[16];
+    if constexpr (EPI == EPI_ENDPOINT) {
+      if (row0 + 16 <= p.R && __all_sync(0xFFFFFFFFu, vj)) {
+        if (p.codes) {
+#pragma unroll
+          for (int q = 0; q < 16; ++q)
+            z[q] = v[q] + pay.c[q] * __shfl_sync(0xFFFFFFFFu, pay.s, q);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 16; ++q) z[q] = v[q];
+        }
+        if (p.Y) {
+          float* zp = p.Y + (int64_t)row0 * p.ldy + j;
+#pragma unroll
+          for (int q = 0; q < 16; ++q, zp += p.ldy) *zp = z[q];
+        }
+        if (!p.seg_stats) return;
+        const float mk = warp_reduce_scatter16(z, MaxOp{}, lane);
+        float e[16];
+        const float l2t = p.inv_tau * kLog2eF;
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+          e[q] = ex2_approx((z[q] - __shfl_sync(0xFFFFFFFFu, mk, 2 * q)) * l2t);
+        const float sk = warp_reduce_scatter16(e, SumOp{}, lane);
+        if (!(lane & 1))
+          p.seg_stats[(int64_t)(row0 + kr) * p.nseg + seg] = make_float2(mk, sk);
+        return;
+      }
+    }
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
       const float sq = __shfl_sync(0xFFFFFFFFu, pay.s, q);
@@ -1044,8 +1109,13 @@ tc_kernel(const __grid_constant__ WMaps wm,
       // the tile from the stored partials.
       constexpr int kMaxC = 8;
       int c0 = 0, C = 1, cnt = 0;
-      bool fin = false, known_last = false, pre_ok = false;
-      float pre[16];                   // two contributors: the other's first chunk
+      bool fin = false, known_last = false;
+      // two or three contributors: the others' partials of the next chunk
+      // (the finisher is the last but one, so pa comes before and pb after
+      // its own part with three, pa after it with two)
+      // (the transposed and the fused epilogues have no registers for them)
+      constexpr bool kParts = EPI == EPI_CLOUD || EPI == EPI_ENDPOINT;
+      float pa[kParts ? 16 : 1], pb[kParts ? 16 : 1];
       if (!whole) {
         cnt = ((tile * 4 + quad) * kEpiGroups + grp) * (PAIR ? 2 : 1) + half;
         c0 = (int)cta_of((long long)tile * p.KB, p.T, G);
@@ -1070,17 +1140,26 @@ tc_kernel(const __grid_constant__ WMaps wm,
         if (lane == 0) arrived = ptx::ld_acquire_gpu(&p.counters[cnt]);
         known_last = __shfl_sync(0xFFFFFFFFu, arrived, 0) == C - 1;
         __syncwarp();
-        // (cloud only: the endpoint epilogue's payload registers leave no
-        // room, and its short hidden dimension mostly gives whole tiles)
-        if (EPI == EPI_CLOUD && known_last && C == 2 && grp < nhc) {
-          const int hf = grp / nch, ch = grp - hf * nch;
-          const float* pc = p.P + (size_t)slot_of(1) * BN * TM + (size_t)ch * 16 * TM +
-                            hf * 128 + quad * 32 + lane;
-#pragma unroll
-          for (int q = 0; q < 16; ++q) pre[q] = __ldcg(pc + (size_t)q * TM);
-          pre_ok = true;
-        }
       }
+      auto load_parts = [&](int hc) {
+        const int hf = hc / nch, ch = hc - hf * nch;
+        const size_t o = (size_t)ch * 16 * TM + hf * 128 + quad * 32 + lane;
+        if constexpr (kParts) {
+          const float* p0 = p.P + (size_t)slot_of(C == 2 ? 1 : 0) * BN * TM + o;
+#pragma unroll
+          for (int q = 0; q < 16; ++q) pa[q] = __ldcg(p0 + q * TM);
+          if (C == 3) {
+            const float* p1 = p.P + (size_t)slot_of(2) * BN * TM + o;
+#pragma unroll
+            for (int q = 0; q < 16; ++q) pb[q] = __ldcg(p1 + q * TM);
+          }
+        }
+      };
+      // (arrived before the accumulator is ready: the first chunk's are
+      // fetched while the MMAs finish)
+      const bool parts = kParts && (C == 2 || C == 3);
+      bool pre_ok = known_last && parts && grp < nhc;
+      if (pre_ok) load_parts(grp);
       int ok = 1;
       if (lane == 0)
         ok = !*s_abort && ptx::mbar_wait(&tfull[acc], fph[acc], limit);
@@ -1105,6 +1184,7 @@ tc_kernel(const __grid_constant__ WMaps wm,
         known_last = __shfl_sync(0xFFFFFFFFu, arrived, 0) == C - 1;
         __syncwarp();
       }
+      if (known_last && parts && !pre_ok && grp < nhc) load_parts(grp);
       ptx::tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) +
                              (uint32_t)(acc * kHalves * BN);
@@ -1123,7 +1203,21 @@ tc_kernel(const __grid_constant__ WMaps wm,
           finish_rm<EPI>(p, v1, r_rm, t * 256 + s1 * 32, rp[a + 1], rq_rm);
         }
       }
-      for (int hc = grp; hc < (rm ? 0 : nhc); hc += kEpiGroups) {
+      // a split tile of two or three contributors: its partials a chunk ahead
+      const bool by_parts = known_last && parts;
+      if constexpr (kParts) {
+        for (int hc = grp; hc < (by_parts ? nhc : 0); hc += kEpiGroups) {
+          const int hf = hc / nch, ch = hc - hf * nch;
+          if constexpr (lane_pay) load_payload<EPI>(p, rb * BN + ch * 16, J(hf), lane, pay);
+          float v[16];
+          ptx::tmem_ld16(taddr + hf * BN + ch * 16, v);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) v[q] = C == 2 ? v[q] + pa[q] : (pa[q] + v[q]) + pb[q];
+          if (hc + kEpiGroups < nhc) load_parts(hc + kEpiGroups);
+          finish(v, hf, ch);
+        }
+      }
+      for (int hc = grp; hc < (rm || by_parts ? 0 : nhc); hc += kEpiGroups) {
         const int hf = hc / nch, ch = hc - hf * nch;
         const int i = hf * 128 + quad * 32 + lane;
         float v[16];
@@ -1152,19 +1246,14 @@ tc_kernel(const __grid_constant__ WMaps wm,
           const int me = unit - c0;
           const size_t o = (size_t)ch * 16 * TM + i;
           float s[16];
-          if (pre_ok && hc == grp) {       // two contributors, the other's part prefetched
 #pragma unroll
-            for (int q = 0; q < 16; ++q) s[q] = v[q] + pre[q];   // (me == 0)
-          } else {
+          for (int c = 0; c < kMaxC; ++c) {
+            if (c < C) {
+              const float* pc = p.P + (size_t)slot_of(c) * BN * TM + o;
 #pragma unroll
-            for (int c = 0; c < kMaxC; ++c) {
-              if (c < C) {
-                const float* pc = p.P + (size_t)slot_of(c) * BN * TM + o;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                  const float x = c == me ? v[q] : __ldcg(pc + (size_t)q * TM);
-                  s[q] = c == 0 ? x : s[q] + x;
-                }
+              for (int q = 0; q < 16; ++q) {
+                const float x = c == me ? v[q] : __ldcg(pc + (size_t)q * TM);
+                s[q] = c == 0 ? x : s[q] + x;
               }
             }
           }
