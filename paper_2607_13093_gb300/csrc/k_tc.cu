@@ -78,6 +78,17 @@ constexpr float kLog2eF = 1.4426950408889634f;   // exp(d / tau) = 2^(d log2(e) 
 // Kernel instantiations of EPI_ENDPOINT that finish through the per-warp
 // shared-memory transpose (finish_chunk_t) rather than per lane.
 constexpr int EPI_ENDPOINT_T = 3;
+// The two forms of the transposed and (below) the rows-as-M endpoint whose
+// rows of codes start anywhere: the codes are fetched as the aligned words
+// that hold them, one more than the aligned forms need, and put together only
+// where they are used.  (Assembling them at the load, from whatever narrower
+// loads the alignment allows, made every chunk wait for memory, and cost the
+// rows-as-M form 32 scattered byte loads a segment: endpoint call with its
+// draw over 51302 ids x 512, 256 rows 54.8 -> 44.2 us, 512 rows 104.6 -> 70.9;
+// z alone for 320 rows 66.3 -> 62.9.  The extra registers cost the aligned
+// shapes up to 11 %, so these are instantiations of their own.)
+constexpr int EPI_ENDPOINT_TU = 6;
+constexpr int EPI_ENDPOINT_RMU = 7;
 // Rows-as-M instantiations of EPI_ENDPOINT and EPI_FUSED (CTA pairs only):
 // the MMA's M dimension is the hidden-state rows (A = the h planes, 128 rows
 // per CTA) and N the tile's 256 ids (B = the gathered weight rows, 128 per
@@ -167,8 +178,9 @@ struct Segments {
 
 
 // Endpoint payload of one 16-row chunk at this lane's id column j: the int8
-// codes of rows row0..row0+15 (as floats) and, in lane q < 16, the scale of
-// row row0 + q.  The fused endpoint loads the cloud's clipped fp32 partials
+// codes of rows row0..row0+15 (as the bits of an int, converted where they
+// are used: a conversion here would wait for the load) and, in lane q < 16,
+// the scale of row row0 + q.  The fused endpoint loads the cloud's clipped fp32 partials
 // instead, and the quantizer's lift and reciprocal of the row scale.
 // Addresses are clamped into the arrays and every load is issued, so the 16
 // loads go out back to back and can be started a chunk ahead of their use.
@@ -200,11 +212,11 @@ __device__ __forceinline__ void load_payload(const TcParams& p, int row0, int j,
   if (row0 + 16 <= p.R) {
     col += (int64_t)row0 * p.n;
 #pragma unroll
-    for (int q = 0; q < 16; ++q, col += p.n) pl.c[q] = (float)__ldg(col);
+    for (int q = 0; q < 16; ++q, col += p.n) pl.c[q] = __int_as_float((int)__ldg(col));
   } else {
 #pragma unroll
     for (int q = 0; q < 16; ++q)
-      pl.c[q] = (float)__ldg(col + (int64_t)min(row0 + q, p.R - 1) * p.n);
+      pl.c[q] = __int_as_float((int)__ldg(col + (int64_t)min(row0 + q, p.R - 1) * p.n));
   }
   pl.s = __ldg(p.row_scale + min(row0 + (lane & 15), p.R - 1));
 }
@@ -291,7 +303,7 @@ __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)
         if (p.codes) {
 #pragma unroll
           for (int q = 0; q < 16; ++q)
-            z[q] = v[q] + pay.c[q] * __shfl_sync(0xFFFFFFFFu, pay.s, q);
+            z[q] = v[q] + (float)__float_as_int(pay.c[q]) * __shfl_sync(0xFFFFFFFFu, pay.s, q);
         } else {
 #pragma unroll
           for (int q = 0; q < 16; ++q) z[q] = v[q];
@@ -317,7 +329,7 @@ __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
       const float sq = __shfl_sync(0xFFFFFFFFu, pay.s, q);
-      float cq = pay.c[q];
+      float cq = EPI == EPI_FUSED ? pay.c[q] : (float)__float_as_int(pay.c[q]);
       if constexpr (EPI == EPI_FUSED) {
         // quantize the cloud's clipped partial (Eq. 18) exactly as the
         // quantize kernel does, emit the code, and dequantize it (Eq. 13)
@@ -364,33 +376,35 @@ __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)
 // Used when rows of codes (and of z, where z is stored) are 2-element
 // aligned.  The payload of a chunk does not depend on the accumulator, so it
 // is loaded a chunk ahead (TPay).
+template <bool U>
 struct TPay {
-  uint2 cw[2];     // the 8 codes of this lane's row and ids, per half
-  float sc[2];     // that row's scale, per half (0 past the rows)
+  uint2 cw[2];         // the 8 codes of this lane's row and ids, per half; U: the first ...
+  uint2 hi[U ? 2 : 1]; // ... and the second aligned word that hold them
+  float sc[2];         // that row's scale, per half (0 past the rows)
 };
+template <bool U>
 __device__ __forceinline__ void load_tpay(const TcParams& p, int row0, int j0w, int lane,
-                                          TPay& t) {
+                                          TPay<U>& t) {
   const int q = lane >> 2, seg = lane & 3;
 #pragma unroll
   for (int h8 = 0; h8 < 2; ++h8) {
     t.cw[h8] = make_uint2(0u, 0u);
+    if constexpr (U) t.hi[h8] = make_uint2(0u, 0u);
     t.sc[h8] = 0.f;
     const int r = row0 + h8 * 8 + q;
     const int j = j0w + 8 * seg;
     if (!p.codes || r >= p.R || j >= p.n) continue;
     t.sc[h8] = __ldg(p.row_scale + r);
-    const int8_t* cp = p.codes + (int64_t)r * p.n + j;     // 2-byte aligned
-    const uintptr_t ca = reinterpret_cast<uintptr_t>(cp);
+    const int8_t* cp = p.codes + (int64_t)r * p.n + j;
     if (j + 8 <= p.n) {
-      if ((ca & 7) == 0) {
-        t.cw[h8] = __ldg(reinterpret_cast<const uint2*>(cp));
-      } else if ((ca & 3) == 0) {
-        t.cw[h8].x = __ldg(reinterpret_cast<const unsigned*>(cp));
-        t.cw[h8].y = __ldg(reinterpret_cast<const unsigned*>(cp) + 1);
+      if constexpr (U) {
+        // (an aligned word that holds one of the row's codes is readable)
+        const uintptr_t ca = reinterpret_cast<uintptr_t>(cp);
+        const uint2* wp = reinterpret_cast<const uint2*>(ca & ~(uintptr_t)7);
+        t.cw[h8] = __ldg(wp);
+        if (ca & 7) t.hi[h8] = __ldg(wp + 1);
       } else {
-        const unsigned short* hp = reinterpret_cast<const unsigned short*>(cp);
-        t.cw[h8].x = (unsigned)__ldg(hp) | ((unsigned)__ldg(hp + 1) << 16);
-        t.cw[h8].y = (unsigned)__ldg(hp + 2) | ((unsigned)__ldg(hp + 3) << 16);
+        t.cw[h8] = __ldg(reinterpret_cast<const uint2*>(cp));
       }
     } else {                                   // the row's last ids
       unsigned w[2] = {0u, 0u};
@@ -401,8 +415,25 @@ __device__ __forceinline__ void load_tpay(const TcParams& p, int row0, int j0w, 
     }
   }
 }
+// The 8 codes of row r, ids j .. j + 7.
+template <bool U>
+__device__ __forceinline__ uint2 tpay_codes(const TcParams& p, const TPay<U>& t, int h8, int r,
+                                            int j) {
+  if constexpr (!U) {
+    return t.cw[h8];
+  } else {
+    const unsigned off =
+        j + 8 <= p.n ? ((unsigned)reinterpret_cast<uintptr_t>(p.codes) +
+                        (unsigned)r * (unsigned)p.n + (unsigned)j) & 7u : 0u;
+    unsigned w0 = t.cw[h8].x, w1 = t.cw[h8].y, w2 = t.hi[h8].x;
+    if (off & 4u) { w0 = w1; w1 = w2; w2 = t.hi[h8].y; }
+    const unsigned s = 8u * (off & 3u);
+    return make_uint2(__funnelshift_r(w0, w1, s), __funnelshift_r(w1, w2, s));
+  }
+}
+template <bool U>
 __device__ __forceinline__ void finish_chunk_t(const TcParams& p, const float (&v)[16], int row0,
-                                               int j0w, int lane, float* tb, const TPay& pay) {
+                                               int j0w, int lane, float* tb, const TPay<U>& pay) {
   const int q = lane >> 2, seg = lane & 3;
 #pragma unroll
   for (int h8 = 0; h8 < 2; ++h8) {
@@ -417,10 +448,11 @@ __device__ __forceinline__ void finish_chunk_t(const TcParams& p, const float (&
     const bool rv = r < p.R;
     float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     const float sc = pay.sc[h8];
+    const uint2 cw = tpay_codes<U>(p, pay, h8, r, j);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      x[e] += (float)(int8_t)((pay.cw[h8].x >> (8 * e)) & 0xFF) * sc;
-      x[4 + e] += (float)(int8_t)((pay.cw[h8].y >> (8 * e)) & 0xFF) * sc;
+      x[e] += (float)(int8_t)((cw.x >> (8 * e)) & 0xFF) * sc;
+      x[4 + e] += (float)(int8_t)((cw.y >> (8 * e)) & 0xFF) * sc;
     }
     if (p.Y && rv && j < p.n) {
       float* zp = p.Y + (int64_t)r * p.ldy + j;               // 8-byte aligned
@@ -463,45 +495,70 @@ __device__ __forceinline__ void finish_chunk_t(const TcParams& p, const float (&
 // This lane's row r and one 32-id segment j0 .. j0 + 31 of the tile.  The
 // codes of the segment (32 bytes of row r), loaded before the tile's
 // accumulator is ready.
+template <bool U>
 struct RPay {
-  uint4 c[2];
+  uint4 c[U ? 3 : 2];  // U: the aligned words that hold them
 };
-__device__ __forceinline__ void load_rpay(const TcParams& p, int r, int j0, RPay& q) {
-  q.c[0] = q.c[1] = make_uint4(0u, 0u, 0u, 0u);
+template <bool U>
+__device__ __forceinline__ void load_rpay(const TcParams& p, int r, int j0, RPay<U>& q) {
+#pragma unroll
+  for (int e = 0; e < (U ? 3 : 2); ++e) q.c[e] = make_uint4(0u, 0u, 0u, 0u);
   if (!p.codes || r >= p.R || j0 >= p.n) return;
   const int8_t* cp = p.codes + (int64_t)r * p.n + j0;
-  const uintptr_t a = reinterpret_cast<uintptr_t>(cp);
-  if (j0 + 32 <= p.n && (a & 15) == 0) {
-    q.c[0] = __ldg(reinterpret_cast<const uint4*>(cp));
-    q.c[1] = __ldg(reinterpret_cast<const uint4*>(cp) + 1);
+  if (j0 + 32 <= p.n) {
+    // (an aligned word that holds one of the row's codes is readable)
+    const uintptr_t a = reinterpret_cast<uintptr_t>(cp);
+    const uint4* wp = reinterpret_cast<const uint4*>(U ? a & ~(uintptr_t)15 : a);
+    q.c[0] = __ldg(wp);
+    q.c[1] = __ldg(wp + 1);
+    if constexpr (U) {
+      if (a & 15) q.c[2] = __ldg(wp + 2);
+    }
     return;
   }
+  const int cnt = p.n - j0;                   // the row's last ids
   unsigned w[8];
-  if (j0 + 32 <= p.n && (a & 3) == 0) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) w[e] = __ldg(reinterpret_cast<const unsigned*>(cp) + e);
-  } else {
-    const int cnt = min(32, p.n - j0);
+  for (int e = 0; e < 8; ++e) w[e] = 0u;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) w[e] = 0u;
-#pragma unroll
-    for (int e = 0; e < 32; ++e)
-      if (e < cnt) w[e >> 2] |= ((unsigned)(uint8_t)__ldg(cp + e)) << (8 * (e & 3));
-  }
+  for (int e = 0; e < 32; ++e)
+    if (e < cnt) w[e >> 2] |= ((unsigned)(uint8_t)__ldg(cp + e)) << (8 * (e & 3));
   q.c[0] = make_uint4(w[0], w[1], w[2], w[3]);
   q.c[1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
-__device__ __forceinline__ unsigned rpay_word(const RPay& q, int w) {
-  const uint4 u = q.c[w >> 2];
-  return (w & 3) == 0 ? u.x : (w & 3) == 1 ? u.y : (w & 3) == 2 ? u.z : u.w;
+// The 32 codes of row r from id j0 on, as 8 words.
+template <bool U>
+__device__ __forceinline__ void rpay_words(const TcParams& p, const RPay<U>& q, int r, int j0,
+                                           unsigned (&w)[8]) {
+  if constexpr (!U) {
+    w[0] = q.c[0].x; w[1] = q.c[0].y; w[2] = q.c[0].z; w[3] = q.c[0].w;
+    w[4] = q.c[1].x; w[5] = q.c[1].y; w[6] = q.c[1].z; w[7] = q.c[1].w;
+  } else {
+    const unsigned off =
+        j0 + 32 <= p.n ? ((unsigned)reinterpret_cast<uintptr_t>(p.codes) +
+                          (unsigned)r * (unsigned)p.n + (unsigned)j0) & 15u : 0u;
+    unsigned x[12] = {q.c[0].x, q.c[0].y, q.c[0].z, q.c[0].w, q.c[1].x, q.c[1].y,
+                      q.c[1].z, q.c[1].w, q.c[2].x, q.c[2].y, q.c[2].z, q.c[2].w};
+    if (off & 8u) {
+#pragma unroll
+      for (int e = 0; e < 10; ++e) x[e] = x[e + 2];
+    }
+    if (off & 4u) {
+#pragma unroll
+      for (int e = 0; e < 9; ++e) x[e] = x[e + 1];
+    }
+    const unsigned s = 8u * (off & 3u);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[e] = __funnelshift_r(x[e], x[e + 1], s);
+  }
 }
 // Finish the segment (Eq. 13): z = v + code * s, stored where asked; with the
 // fused endpoint the codes are first quantized from the cloud's clipped
 // partials (Eq. 18) and written out; the segment's softmax statistics
 // (max z, sum of exp((z - max) / tau) over its ids below n) where asked.
-template <int EPI>
+template <int EPI, bool U>
 __device__ __forceinline__ void finish_rm(const TcParams& p, float (&v)[32], int r, int j0,
-                                          const RPay& q, const RowQuant& rq) {
+                                          const RPay<U>& q, const RowQuant& rq) {
   const bool rv = r < p.R;
   const int cnt = rv ? max(0, min(32, p.n - j0)) : 0;   // this row's ids in the segment
   const bool full = cnt == 32;
@@ -540,9 +597,11 @@ __device__ __forceinline__ void finish_rm(const TcParams& p, float (&v)[32], int
     }
   } else {
     if (p.codes) {
+      unsigned cw[8];
+      rpay_words<U>(p, q, r, j0, cw);
 #pragma unroll
       for (int w = 0; w < 8; ++w) {
-        const unsigned wx = rpay_word(q, w) ^ 0x80808080u;
+        const unsigned wx = cw[w] ^ 0x80808080u;
 #pragma unroll
         for (int b = 0; b < 4; ++b) v[4 * w + b] = fmaf(code_f32(wx, b), rq.s, v[4 * w + b]);
       }
@@ -611,7 +670,7 @@ tc_kernel(const __grid_constant__ WMaps wm,
   static_assert(!PAIR || TM == 128, "a pair tile is two CTAs of 128 ids");
   // rows as M: the MMA's A operand is the h planes and B the weights (the
   // same shared-memory stages); pairs of CTAs with 256-row blocks only
-  constexpr bool rm = EPI == EPI_ENDPOINT_RM || EPI == EPI_FUSED_RM;
+  constexpr bool rm = EPI == EPI_ENDPOINT_RM || EPI == EPI_ENDPOINT_RMU || EPI == EPI_FUSED_RM;
   static_assert(!rm || (PAIR && !FP8), "rows as M: bf16 CTA pairs");
   constexpr int kAtomE = FP8 ? kAtomE8 : kAtomK;   // elements per 128-byte atom
   extern __shared__ uint8_t smem_raw[];
@@ -1024,7 +1083,8 @@ tc_kernel(const __grid_constant__ WMaps wm,
       auto ID = [&](int hf) { return (kHalves > 1 && hf) ? idh[kHalves - 1] : idh[0]; };
       // the endpoint through this warp's transpose tile (no per-lane
       // payload registers then)
-      constexpr bool epi_t = EPI == EPI_ENDPOINT_T;
+      constexpr bool epi_t = EPI == EPI_ENDPOINT_T || EPI == EPI_ENDPOINT_TU;
+      constexpr bool kU = EPI == EPI_ENDPOINT_TU || EPI == EPI_ENDPOINT_RMU;
       constexpr bool lane_pay = EPI == EPI_ENDPOINT || EPI == EPI_FUSED;
       float* tb = reinterpret_cast<float*>(base + (size_t)S * stage_bytes + kBarrierArea +
                                            kMaxBoxes * sizeof(int2)) +
@@ -1036,7 +1096,7 @@ tc_kernel(const __grid_constant__ WMaps wm,
       constexpr int kRmSeg = 8 / kEpiGroups;
       const int r_rm = rb * 256 + half * 128 + quad * 32 + lane;
       RowQuant rq_rm{0.f, 1.f, 0.f};
-      RPay rp[kRmSeg];
+      RPay<kU> rp[kRmSeg];
       if constexpr (rm) {
         if (r_rm < p.R) {
           if constexpr (EPI == EPI_FUSED_RM) {
@@ -1053,10 +1113,10 @@ tc_kernel(const __grid_constant__ WMaps wm,
             rq_rm.s = __ldg(p.row_scale + r_rm);
           }
         }
-        if constexpr (EPI == EPI_ENDPOINT_RM) {
+        if constexpr (EPI != EPI_FUSED_RM) {
 #pragma unroll
           for (int a = 0; a < kRmSeg; ++a)
-            load_rpay(p, r_rm, t * 256 + (grp + a * kEpiGroups) * 32, rp[a]);
+            load_rpay<kU>(p, r_rm, t * 256 + (grp + a * kEpiGroups) * 32, rp[a]);
         }
       }
       if constexpr (EPI != EPI_CLOUD && !rm) {
@@ -1074,14 +1134,14 @@ tc_kernel(const __grid_constant__ WMaps wm,
       // the one being finished (tq[a]: chunk hc + (a + 1) kEpiGroups): a
       // chunk's work is shorter than a load's latency under the kernel's
       // own traffic
-      constexpr int kTAhead = 3;
-      TPay tpay, tq[kTAhead];
+      constexpr int kTAhead = kU ? 2 : 3;
+      TPay<kU> tpay, tq[kTAhead];
       if (epi_t && whole) {
 #pragma unroll
         for (int a = 0; a <= kTAhead; ++a) {
           const int hn = grp + a * kEpiGroups;
           if (hn < nhc)
-            load_tpay(p, rb * BN + (hn % nch) * 16, J(hn / nch) - lane, lane,
+            load_tpay<kU>(p, rb * BN + (hn % nch) * 16, J(hn / nch) - lane, lane,
                       a == 0 ? tpay : tq[a - 1]);
         }
       }
@@ -1090,8 +1150,8 @@ tc_kernel(const __grid_constant__ WMaps wm,
         if constexpr (rm) {
           // (rows as M takes whole tiles only)
         } else if constexpr (epi_t) {
-          if (!whole) load_tpay(p, rb * BN + ch * 16, J(hf) - lane, lane, tpay);
-          finish_chunk_t(p, vv, rb * BN + ch * 16, J(hf) - lane, lane, tb, tpay);
+          if (!whole) load_tpay<kU>(p, rb * BN + ch * 16, J(hf) - lane, lane, tpay);
+          finish_chunk_t<kU>(p, vv, rb * BN + ch * 16, J(hf) - lane, lane, tb, tpay);
         } else {
           finish_chunk<EPI>(p, vv, rb * BN + ch * 16, J(hf), VJ(hf), ID(hf), lane,
                             segb + hf * 4 + quad, pay);
@@ -1199,8 +1259,8 @@ tc_kernel(const __grid_constant__ WMaps wm,
           const int s0 = grp + a * kEpiGroups, s1 = s0 + kEpiGroups;
           float v0[32], v1[32];
           ptx::tmem_ld32x2(taddr + (uint32_t)(s0 * 32), taddr + (uint32_t)(s1 * 32), v0, v1);
-          finish_rm<EPI>(p, v0, r_rm, t * 256 + s0 * 32, rp[a], rq_rm);
-          finish_rm<EPI>(p, v1, r_rm, t * 256 + s1 * 32, rp[a + 1], rq_rm);
+          finish_rm<EPI, kU>(p, v0, r_rm, t * 256 + s0 * 32, rp[a], rq_rm);
+          finish_rm<EPI, kU>(p, v1, r_rm, t * 256 + s1 * 32, rp[a + 1], rq_rm);
         }
       }
       // a split tile of two or three contributors: its partials a chunk ahead
@@ -1225,12 +1285,12 @@ tc_kernel(const __grid_constant__ WMaps wm,
         if (whole) {
           Payload nxt;
           const int hn = hc + kEpiGroups;
-          TPay tnxt;
+          TPay<kU> tnxt;
           if constexpr (lane_pay)
             if (hn < nhc) load_payload<EPI>(p, rb * BN + (hn % nch) * 16, J(hn / nch), lane, nxt);
           const int ht = hc + (kTAhead + 1) * kEpiGroups;
           if (epi_t && ht < nhc)
-            load_tpay(p, rb * BN + (ht % nch) * 16, J(ht / nch) - lane, lane, tnxt);
+            load_tpay<kU>(p, rb * BN + (ht % nch) * 16, J(ht / nch) - lane, lane, tnxt);
           finish(v, hf, ch);
           if constexpr (lane_pay) pay = nxt;
           if constexpr (epi_t) {
@@ -2023,6 +2083,9 @@ cudaError_t launch_tc(const GatherGemm& g, const TcPlan& pl, void* scratch,
   prm.P = P; prm.counters = counters;
   prm.status = g.status; prm.spin_limit = spin_limit; prm.finish_wait = g.finish_wait;
 
+  // rows of codes that start on the words the aligned forms load
+  const uintptr_t cal = reinterpret_cast<uintptr_t>(g.codes) | (uintptr_t)(unsigned)g.n;
+  const bool c8 = (cal & 7) == 0, c16 = (cal & 15) == 0;
   const bool hilo2 = pl.hilo == 2;
   if (pl.pair && fp8) {
     // (two planes a stage, in one group or two)
@@ -2034,6 +2097,9 @@ cudaError_t launch_tc(const GatherGemm& g, const TcPlan& pl, void* scratch,
     if (g.epilogue == EPI_FUSED)
       return gather ? launch_inst<2, true, EPI_FUSED_RM, false, 128, true>(mw, mh, prm, pl, st)
                     : launch_inst<2, false, EPI_FUSED_RM, false, 128, true>(mw, mh, prm, pl, st);
+    if (g.codes && !c16)
+      return gather ? launch_inst<2, true, EPI_ENDPOINT_RMU, false, 128, true>(mw, mh, prm, pl, st)
+                    : launch_inst<2, false, EPI_ENDPOINT_RMU, false, 128, true>(mw, mh, prm, pl, st);
     return gather ? launch_inst<2, true, EPI_ENDPOINT_RM, false, 128, true>(mw, mh, prm, pl, st)
                   : launch_inst<2, false, EPI_ENDPOINT_RM, false, 128, true>(mw, mh, prm, pl, st);
   }
@@ -2041,6 +2107,9 @@ cudaError_t launch_tc(const GatherGemm& g, const TcPlan& pl, void* scratch,
     if (g.epilogue == EPI_FUSED)
       return gather ? launch_inst<2, true, EPI_FUSED, false, 128, true>(mw, mh, prm, pl, st)
                     : launch_inst<2, false, EPI_FUSED, false, 128, true>(mw, mh, prm, pl, st);
+    if (et && g.codes && !c8)
+      return gather ? launch_inst<2, true, EPI_ENDPOINT_TU, false, 128, true>(mw, mh, prm, pl, st)
+                    : launch_inst<2, false, EPI_ENDPOINT_TU, false, 128, true>(mw, mh, prm, pl, st);
     if (et)
       return gather ? launch_inst<2, true, EPI_ENDPOINT_T, false, 128, true>(mw, mh, prm, pl, st)
                     : launch_inst<2, false, EPI_ENDPOINT_T, false, 128, true>(mw, mh, prm, pl, st);
@@ -2069,6 +2138,9 @@ cudaError_t launch_tc(const GatherGemm& g, const TcPlan& pl, void* scratch,
     if (g.epilogue == EPI_FUSED)
       return gather ? launch_inst<2, true, EPI_FUSED, false, 256>(mw, mh, prm, pl, st)
                     : launch_inst<2, false, EPI_FUSED, false, 256>(mw, mh, prm, pl, st);
+    if (et && g.codes && !c8)
+      return gather ? launch_inst<2, true, EPI_ENDPOINT_TU, false, 256>(mw, mh, prm, pl, st)
+                    : launch_inst<2, false, EPI_ENDPOINT_TU, false, 256>(mw, mh, prm, pl, st);
     if (et)
       return gather ? launch_inst<2, true, EPI_ENDPOINT_T, false, 256>(mw, mh, prm, pl, st)
                     : launch_inst<2, false, EPI_ENDPOINT_T, false, 256>(mw, mh, prm, pl, st);
@@ -2090,6 +2162,9 @@ cudaError_t launch_tc(const GatherGemm& g, const TcPlan& pl, void* scratch,
   if (g.epilogue == EPI_FUSED)
     return gather ? launch_inst<2, true, EPI_FUSED>(mw, mh, prm, pl, st)
                   : launch_inst<2, false, EPI_FUSED>(mw, mh, prm, pl, st);
+  if (et && g.codes && !c8)
+    return gather ? launch_inst<2, true, EPI_ENDPOINT_TU>(mw, mh, prm, pl, st)
+                  : launch_inst<2, false, EPI_ENDPOINT_TU>(mw, mh, prm, pl, st);
   if (et)
     return gather ? launch_inst<2, true, EPI_ENDPOINT_T>(mw, mh, prm, pl, st)
                   : launch_inst<2, false, EPI_ENDPOINT_T>(mw, mh, prm, pl, st);

@@ -1,0 +1,44 @@
+"""Payloads whose rows of codes start anywhere: the transposed and the
+rows-as-M endpoint fetch them as the aligned words that hold them.  The same
+bits for every base address, and the oracle's values.  Needs a GPU (marked
+gpu)."""
+import pytest
+import torch
+
+from paper_2607_13093_gb300 import workloads as wl
+from _parity import check_endpoint
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+# 160 rows: ids as M through the transpose (an even number of ids); 250: rows
+# as M.  Ids: whole 32-id segments, and last segments of 1, 8, 10 and 31 ids;
+# divisible by 16, 8, 4, 2 and 1
+@pytest.mark.parametrize("rows,n", [(160, 1024), (160, 1032), (160, 1034), (160, 1036), (250, 1024),
+                                    (250, 1032), (250, 1034), (250, 1055), (250, 1025)])
+def test_code_rows_at_any_address(rows, n):
+    from paper_2607_13093_gb300 import build_lib
+    build_lib.build()
+    from paper_2607_13093_gb300 import sph
+    ctx = sph.Context(0)
+    w = wl.make_workload(V=2000, d=160, d_l=64, rows=rows, n_keep=n, seed=n, device=DEV, tau=0.9)
+    pc, ps = wl.make_payload(rows, n, seed=5, device=DEV)
+    check_endpoint(ctx, w, pc.cpu(), ps.cpu(), unstored=False)
+    outs = []
+    for shift in (0, 1, 2, 4, 6, 8, 13, 15):
+        buf = torch.full((rows * n + 32,), 77, dtype=torch.int8, device=DEV)
+        codes = buf[shift:shift + rows * n].view(rows, n)
+        codes.copy_(pc)
+        z = torch.empty(rows, n, device=DEV)
+        ctx.fuse_sample(codes, ps, w.h_local, w.W_l, keep_ids=w.keep_ids, draw=False,
+                        fused_logits_out=z)
+        t = ctx.fuse_sample(codes, ps, w.h_local, w.W_l, keep_ids=w.keep_ids, temperature=0.9,
+                            seed=3, offset=shift)
+        g = ctx.fuse_sample(codes, ps, w.h_local, w.W_l, keep_ids=w.keep_ids, temperature=0.0)
+        ctx.sync()
+        outs.append((z, g))
+        assert t.min() >= 0
+    for z, g in outs[1:]:
+        assert torch.equal(z, outs[0][0]) and torch.equal(g, outs[0][1])
+    ctx.close()
