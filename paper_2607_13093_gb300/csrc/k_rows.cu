@@ -495,6 +495,131 @@ sample_rows_kernel(const ZRows zr, int n, const float2* __restrict__ stats,
   }
 }
 
+__device__ __forceinline__ int warp_min_int(int v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v = min(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+  return v;
+}
+
+// The lowest segment holding the row maximum (from its statistics), then the
+// lowest id in it whose z equals the segment's largest z (the maximum
+// itself where z is stored); all lanes return it.
+template <class ZR>
+__device__ __forceinline__ int warp_argmax(const ZR& z, int n, const float2* st, int nseg,
+                                           int lane) {
+  float M = -INFINITY;
+  int sb = nseg;
+  for (int s = lane; s < nseg; s += 32) {
+    const float m = st[s].x;
+    if (m > M) { M = m; sb = s; }
+  }
+  const float Mw = warp_max(M);
+  if (!(Mw > -INFINITY)) return 0;
+  const int seg = warp_min_int(M == Mw ? sb : nseg);
+  const int j = seg * kSeg + lane;
+  const float zj = j < n ? z(j) : -INFINITY;
+  const float mz = warp_max(zj);
+  const unsigned hit = __ballot_sync(0xFFFFFFFFu, j < n && zj == mz);
+  return hit ? seg * kSeg + __ffs(hit) - 1 : min(seg * kSeg, n - 1);
+}
+
+// What the statistics pass does with a chunk, for a warp that has just one:
+// the chunk at z (`left` of its row's ids from there on) through the warp's
+// tile tb; this lane's segment's (max, sum of exp), the same tree of sums.
+// (The pass itself keeps its own text: with this function called from its
+// loop, 3 rows x 32000 ids took 18.98 us instead of 18.38.)
+__device__ __forceinline__ float2 chunk_segment_stats(const float* __restrict__ z, int left,
+                                                      float* tb, float l2t, int lane) {
+  if (left >= kSeg * kSeg && ((reinterpret_cast<uintptr_t>(z) & 15) == 0)) {
+#pragma unroll
+    for (int q = 0; q < kSeg / 4; ++q) {
+      const float4 t = __ldcs(reinterpret_cast<const float4*>(z) + q * 32 + lane);
+      *reinterpret_cast<float4*>(tb + (q * 4 + (lane >> 3)) * kSegRow + 4 * (lane & 7)) = t;
+    }
+  } else {
+#pragma unroll 8
+    for (int q = 0; q < kSeg; ++q) {
+      const int e = q * 32 + lane;
+      tb[q * kSegRow + lane] = e < left ? __ldcs(z + e) : -INFINITY;
+    }
+  }
+  __syncwarp();
+  float v[kSeg];
+#pragma unroll
+  for (int m = 0; m < kSeg / 4; ++m) {
+    const float4 t = *reinterpret_cast<const float4*>(tb + lane * kSegRow + 4 * m);
+    v[4 * m] = t.x; v[4 * m + 1] = t.y; v[4 * m + 2] = t.z; v[4 * m + 3] = t.w;
+  }
+  float t[kSeg / 2];
+#pragma unroll
+  for (int q = 0; q < kSeg / 2; ++q) t[q] = fmaxf(v[2 * q], v[2 * q + 1]);
+#pragma unroll
+  for (int w = kSeg / 4; w >= 1; w >>= 1)
+#pragma unroll
+    for (int q = 0; q < w; ++q) t[q] = fmaxf(t[2 * q], t[2 * q + 1]);
+  const float m = t[0];
+  float sum = 0.f;
+  if (m > -INFINITY) {
+    // exp of -inf (ids past n) is 0
+#pragma unroll
+    for (int q = 0; q < kSeg / 2; ++q)
+      t[q] = exp_tau(v[2 * q] - m, l2t) + exp_tau(v[2 * q + 1] - m, l2t);
+#pragma unroll
+    for (int w = kSeg / 4; w >= 1; w >>= 1)
+#pragma unroll
+      for (int q = 0; q < w; ++q) t[q] = t[2 * q] + t[2 * q + 1];
+    sum = t[0];
+  }
+  return make_float2(m, sum);
+}
+
+// The draw of a short stored row in one launch: the block's warps make the
+// row's segment and chunk statistics in shared memory -- the same reductions,
+// and so the same values, as the statistics pass -- and warp 0 draws (greedy:
+// takes the first maximum).  Such a call is bound by its launches and the
+// latency of each; this saves one of three and the statistics' way through
+// memory.  Token calls of d_l 64 with it and without: 1 row x 2048 ids 5.5 us
+// and 6.7, 3 x 8192 9.8 and 11.4, 16 x 8192 21.4 and 23.0.  A chunk a warp at
+// most: with two, 3 x 16382 ids took 14.8 us instead of 14.6.  16 rows at
+// most: 300 x 2048 took 193 us instead of 174.
+constexpr int kShortChunks = kWarps;
+constexpr int kShortRows = 16;
+__global__ void __launch_bounds__(kWarps * 32)
+sample_short_kernel(const ZRowsStored zr, int n, const int32_t* __restrict__ ids, float inv_tau,
+                    uint64_t seed, uint64_t offset, int greedy, int32_t* __restrict__ tokens) {
+  __shared__ __align__(16) float tile[kWarps][kSeg * kSegRow];
+  __shared__ float2 s_seg[kShortChunks * kSeg];
+  __shared__ float2 s_cst[kShortChunks];
+  ptx::griddep_wait();
+  ptx::griddep_launch_dependents();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r = blockIdx.x;
+  const int nseg = (n + kSeg - 1) / kSeg, nchunk = (nseg + kSeg - 1) / kSeg;
+  const ZRowStored z = zr.row(r);
+  if (warp < nchunk) {
+    const int j0 = warp * kSeg * kSeg;          // the chunk's first id
+    const float2 st = chunk_segment_stats(z.z + j0, n - j0, tile[warp], inv_tau * kLog2e, lane);
+    s_seg[warp * kSeg + lane] = st;
+    const float Mc = warp_max(st.x);
+    const float Sc = warp_sum(seg_weight(st, Mc, inv_tau));
+    if (lane == 0) s_cst[warp] = make_float2(Mc, Sc);
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  int j;
+  if (greedy) {
+    j = warp_argmax(z, n, s_seg, nseg, lane);
+  } else {
+    const float M = stats_max(s_cst, nchunk, lane);
+    const StatsWeight cw{s_cst, M, inv_tau};
+    const StatsWeight sw{s_seg, M, inv_tau};
+    const ExpWeight ew{z, M, inv_tau};
+    const float u = philox_uniform(seed, (uint32_t)r, 0u, offset);
+    warp_draw(nchunk, nseg, n, cw, sw, ew, u, lane, j);
+  }
+  if (lane == 0) tokens[r] = ids ? ids[j] : j;
+}
+
 // ---------------------------------------------------------------------------
 // Gumbel-max sampling (the alternative single-pass sampler): the first index
 // of the largest z_j / tau - log(-log u_j) is a draw from softmax(z / tau).
@@ -562,34 +687,6 @@ gumbel_rows_kernel(const float* __restrict__ Z, int n, const int32_t* __restrict
 // ---------------------------------------------------------------------------
 // greedy decoding (temperature 0): the first id of the row maximum
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int warp_min_int(int v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v = min(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-  return v;
-}
-
-// The lowest segment holding the row maximum (from its statistics), then the
-// lowest id in it whose z equals the segment's largest z (the maximum
-// itself where z is stored); all lanes return it.
-template <class ZR>
-__device__ __forceinline__ int warp_argmax(const ZR& z, int n, const float2* st, int nseg,
-                                           int lane) {
-  float M = -INFINITY;
-  int sb = nseg;
-  for (int s = lane; s < nseg; s += 32) {
-    const float m = st[s].x;
-    if (m > M) { M = m; sb = s; }
-  }
-  const float Mw = warp_max(M);
-  if (!(Mw > -INFINITY)) return 0;
-  const int seg = warp_min_int(M == Mw ? sb : nseg);
-  const int j = seg * kSeg + lane;
-  const float zj = j < n ? z(j) : -INFINITY;
-  const float mz = warp_max(zj);
-  const unsigned hit = __ballot_sync(0xFFFFFFFFu, j < n && zj == mz);
-  return hit ? seg * kSeg + __ffs(hit) - 1 : min(seg * kSeg, n - 1);
-}
-
 // One warp per row: vocabulary ids into tokens and/or compact indices.
 template <class ZRows>
 __global__ void __launch_bounds__(kWarps * 32)
@@ -904,6 +1001,18 @@ cudaError_t launch_sample_rows(const ZSource& zs, int rows, int n, const float2*
   if (!zs.h || !zs.W || zs.K < 1 || (zs.codes && !zs.row_scale)) return cudaErrorInvalidValue;
   return sample_rows_with(ZRowsRecomputed{zs, n}, rows, n, stats, nseg, ids, inv_tau, seed,
                           offset, tokens, st);
+}
+
+bool sample_is_short(int rows, int n) {
+  return rows <= kShortRows && chunk_count(seg_count(n)) <= kShortChunks;
+}
+
+cudaError_t launch_sample_short(const float* Z, int rows, int n, const int32_t* ids, float inv_tau,
+                                uint64_t seed, uint64_t offset, int32_t* tokens, cudaStream_t st,
+                                int greedy) {
+  if (rows < 1 || !sample_is_short(rows, n)) return cudaErrorNotSupported;
+  return launch_pdl(sample_short_kernel, dim3(rows), dim3(kWarps * 32), 0, st, ZRowsStored{Z, n},
+                    n, ids, inv_tau, seed, offset, greedy, tokens);
 }
 
 cudaError_t launch_sample_made_stats(const ZSource& zs, int rows, int n, const float2* stats,

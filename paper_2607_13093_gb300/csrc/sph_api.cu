@@ -477,6 +477,10 @@ sph_status endpoint_draw(sph_ctx* ctx, sph::GatherGemm& gg, Carve& c, float temp
   if (st || fuse_only) return st;
   if (gumbel) return draw_gumbel();
   return launch_status(ctx, traced(ctx, SPH_PROF_SAMPLE, [&] {
+                         if (sph::sample_is_short(rows, n_keep))
+                           return sph::launch_sample_short(Z, rows, n_keep, keep_ids, gg.inv_tau,
+                                                           seed, offset, tokens, ctx->stream,
+                                                           greedy);
                          cudaError_t e = sph::launch_seg_stats(Z, rows, n_keep,
                                                                gg.inv_tau, stats,
                                                                cstats, ctx->sm_count,

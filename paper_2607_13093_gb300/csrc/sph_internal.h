@@ -273,6 +273,12 @@ cudaError_t launch_sample_made_stats(const ZSource& zs, int rows, int n, const f
                                      float inv_tau, uint64_t seed, uint64_t offset,
                                      int sm_count, int32_t* tokens, cudaStream_t st,
                                      int greedy);
+// One draw per row (greedy: the argmax) of a short stored row, statistics and
+// draw in one launch (sample_is_short: at most 16 rows of at most 8192 ids).
+bool sample_is_short(int rows, int n);
+cudaError_t launch_sample_short(const float* Z, int rows, int n, const int32_t* ids, float inv_tau,
+                                uint64_t seed, uint64_t offset, int32_t* tokens, cudaStream_t st,
+                                int greedy);
 int sample_max_n();
 int verify_max_k();
 
