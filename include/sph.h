@@ -149,16 +149,18 @@ typedef enum sph_option {
                                repeated or out-of-range ids.  0 (default):
                                the ids are a precondition, not checked.    */
   SPH_OPT_TC_PAIR = 11,     /* CTA pairs for the tensor-core contractions
-                               (the cloud's with bf16 weights, and the
-                               endpoint's; clusters of two CTAs, tcgen05
-                               .cta_group::2): each 256-id tile is one M = 256
+                               (the cloud's and the endpoint's; clusters of
+                               two CTAs, tcgen05 .cta_group::2): each 256-id tile is one M = 256
                                MMA over both CTAs' shared memory, each CTA
                                loading 128 ids of the weights and half of the
                                hidden-state rows.  0 (default): where the row
-                               blocks are long (bf16 weights; >= 128 rows
-                               for the cloud, >= 192 for the endpoint);
-                               1: always (SPH_ERR_
-                               UNSUPPORTED where pairs cannot be scheduled);
+                               blocks are long (cloud: >= 128 rows with bf16
+                               weights; with e4m3 weights >= 224, or >= 160
+                               for bf16-rounded activations, where whole
+                               tiles are scheduled either way; endpoint:
+                               >= 192);
+                               1: always (SPH_ERR_UNSUPPORTED where pairs
+                               cannot be scheduled);
                                2: never.  The results are the fp32 sums of
                                the same products either way.               */
   SPH_OPT_SPLIT_QUANTIZE = 10, /* sph_split_step with one payload chunk: 0
@@ -281,7 +283,8 @@ typedef struct sph_plan {
   int32_t tensor_core;      /* 1: tcgen05 kernel; 0: CUDA-core GEMV        */
   int32_t row_blocks;       /* hidden-state row blocks (tensor core)       */
   int32_t block_rows;       /* rows per row block (a multiple of 16)       */
-  int32_t tile_ids;         /* kept ids per vocabulary tile: 128 or 256    */
+  int32_t tile_ids;         /* kept ids per vocabulary tile: 128 or 256
+                               (32..128 on the endpoint's few-row kernel)  */
   int32_t tiles;            /* row blocks x vocabulary tiles               */
   int32_t k_blocks;         /* pipeline stages per tile (hidden dimension) */
   int32_t stages;           /* shared-memory pipeline depth                */

@@ -299,7 +299,8 @@ __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)
   } else {
     float z[16];
     if constexpr (EPI == EPI_ENDPOINT) {
-      if (row0 + 16 <= p.R && __all_sync(0xFFFFFFFFu, vj)) {
+      if (j - lane + 32 <= p.n) {
+        const int nr = p.R - row0;            // rows of the chunk that exist
         if (p.codes) {
 #pragma unroll
           for (int q = 0; q < 16; ++q)
@@ -311,7 +312,8 @@ __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)
         if (p.Y) {
           float* zp = p.Y + (int64_t)row0 * p.ldy + j;
 #pragma unroll
-          for (int q = 0; q < 16; ++q, zp += p.ldy) *zp = z[q];
+          for (int q = 0; q < 16; ++q, zp += p.ldy)
+            if (q < nr) *zp = z[q];
         }
         if (!p.seg_stats) return;
         const float mk = warp_reduce_scatter16(z, MaxOp{}, lane);
@@ -321,7 +323,7 @@ __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)
         for (int q = 0; q < 16; ++q)
           e[q] = ex2_approx((z[q] - __shfl_sync(0xFFFFFFFFu, mk, 2 * q)) * l2t);
         const float sk = warp_reduce_scatter16(e, SumOp{}, lane);
-        if (!(lane & 1))
+        if (!(lane & 1) && kr < nr)
           p.seg_stats[(int64_t)(row0 + kr) * p.nseg + seg] = make_float2(mk, sk);
         return;
       }
@@ -505,9 +507,9 @@ __device__ __forceinline__ void load_rpay(const TcParams& p, int r, int j0, RPay
   for (int e = 0; e < (U ? 3 : 2); ++e) q.c[e] = make_uint4(0u, 0u, 0u, 0u);
   if (!p.codes || r >= p.R || j0 >= p.n) return;
   const int8_t* cp = p.codes + (int64_t)r * p.n + j0;
-  if (j0 + 32 <= p.n) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(cp);
+  if (j0 + 32 <= p.n && (U || (a & 15) == 0)) {
     // (an aligned word that holds one of the row's codes is readable)
-    const uintptr_t a = reinterpret_cast<uintptr_t>(cp);
     const uint4* wp = reinterpret_cast<const uint4*>(U ? a & ~(uintptr_t)15 : a);
     q.c[0] = __ldg(wp);
     q.c[1] = __ldg(wp + 1);
@@ -516,8 +518,15 @@ __device__ __forceinline__ void load_rpay(const TcParams& p, int r, int j0, RPay
     }
     return;
   }
-  const int cnt = p.n - j0;                   // the row's last ids
   unsigned w[8];
+  if (!U && j0 + 32 <= p.n && (a & 3) == 0) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[e] = __ldg(reinterpret_cast<const unsigned*>(cp) + e);
+    q.c[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    q.c[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    return;
+  }
+  const int cnt = min(32, p.n - j0);
 #pragma unroll
   for (int e = 0; e < 8; ++e) w[e] = 0u;
 #pragma unroll
@@ -1173,8 +1182,10 @@ tc_kernel(const __grid_constant__ WMaps wm,
       // two or three contributors: the others' partials of the next chunk
       // (the finisher is the last but one, so pa comes before and pb after
       // its own part with three, pa after it with two)
-      // (the transposed and the fused epilogues have no registers for them)
-      constexpr bool kParts = EPI == EPI_CLOUD || EPI == EPI_ENDPOINT;
+      // (the endpoint's epilogues have no registers for them: with them the
+      // per-lane form spilled 250 bytes, and 32 rows x 12000 ids x 4096 took
+      // 41.9 us instead of 36.0)
+      constexpr bool kParts = EPI == EPI_CLOUD;
       float pa[kParts ? 16 : 1], pb[kParts ? 16 : 1];
       if (!whole) {
         cnt = ((tile * 4 + quad) * kEpiGroups + grp) * (PAIR ? 2 : 1) + half;
@@ -1268,7 +1279,6 @@ tc_kernel(const __grid_constant__ WMaps wm,
       if constexpr (kParts) {
         for (int hc = grp; hc < (by_parts ? nhc : 0); hc += kEpiGroups) {
           const int hf = hc / nch, ch = hc - hf * nch;
-          if constexpr (lane_pay) load_payload<EPI>(p, rb * BN + ch * 16, J(hf), lane, pay);
           float v[16];
           ptx::tmem_ld16(taddr + hf * BN + ch * 16, v);
 #pragma unroll
@@ -2097,7 +2107,14 @@ cudaError_t launch_tc(const GatherGemm& g, const TcPlan& pl, void* scratch,
     if (g.epilogue == EPI_FUSED)
       return gather ? launch_inst<2, true, EPI_FUSED_RM, false, 128, true>(mw, mh, prm, pl, st)
                     : launch_inst<2, false, EPI_FUSED_RM, false, 128, true>(mw, mh, prm, pl, st);
-    if (g.codes && !c16)
+    // payload rows off 16 bytes: as aligned words where the contraction is too
+    // short to hide the epilogue, else byte by byte, which leaves the copies
+    // undisturbed under a long one.  Words / bytes, us: 256 rows x 51302 ids
+    // 38.0 / 51.8 at K = 256, 47.3 / 59.4 at 512, 71.5 / 77.2 at 1024, 94.7 /
+    // 90.7 at 1536, 116.0 / 110.5 at 2048; x 7001 ids (less than a tile a
+    // pair) 26.9 / 28.3 at 512, 39.1 / 38.2 at 1024.
+    const bool words = g.K <= 512 || (g.K <= 1024 && pl.NT * pl.RB > pl.G / 2);
+    if (g.codes && !c16 && words)
       return gather ? launch_inst<2, true, EPI_ENDPOINT_RMU, false, 128, true>(mw, mh, prm, pl, st)
                     : launch_inst<2, false, EPI_ENDPOINT_RMU, false, 128, true>(mw, mh, prm, pl, st);
     return gather ? launch_inst<2, true, EPI_ENDPOINT_RM, false, 128, true>(mw, mh, prm, pl, st)

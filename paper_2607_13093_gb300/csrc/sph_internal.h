@@ -152,9 +152,9 @@ struct TcPlan {
 // max_bn = most hidden-state rows per tile (0 = automatic); tile_m =
 // vocabulary rows per tile (128, 256 = two M = 128 halves, 0 = automatic);
 // pair_mode = CTA pairs on 256-id tiles: 0 never, 1 where the row blocks are
-// long enough (bf16 weights), 2 always; max_pairs caps the pairs (0: no cap); rm_mode = the endpoint on
-// pairs with rows as M: 0 where the 256-row blocks pad little, 1 always
-// (where the call pairs), 2 never.
+// long enough (SPH_OPT_TC_PAIR has the rows), 2 always; max_pairs caps the
+// pairs (0: no cap); rm_mode = the endpoint on pairs with rows as M: 0 where
+// the 256-row blocks pad little, 1 always (where the call pairs), 2 never.
 TcPlan tc_plan(int rows, int n, int K, int act_bf16, int sm_count, int endpoint,
                int schedule, int max_stages, int block_k, int gather, int fp8, int max_bn,
                int tile_m, int pair_mode = 0, int max_pairs = 0, int rm_mode = 0);

@@ -42,3 +42,21 @@ def test_code_rows_at_any_address(rows, n):
     for z, g in outs[1:]:
         assert torch.equal(z, outs[0][0]) and torch.equal(g, outs[0][1])
     ctx.close()
+
+
+@pytest.mark.parametrize("rows,n,K", [(250, 1034, 512), (250, 1034, 520), (250, 1034, 1024),
+                                      (256, 25602, 1024), (256, 25602, 1032), (250, 1055, 2048),
+                                      (4, 1034, 1024), (15, 1024, 2048), (17, 1055, 1024)])
+def test_code_rows_over_long_hidden_dimensions(rows, n, K):
+    # both sides of the lines at which rows off 16 bytes are fetched as words
+    # (512 columns; 1024 with more tiles than CTA pairs), and the per-lane
+    # epilogue's row chunks that are not full, on whole and on split tiles
+    from paper_2607_13093_gb300 import build_lib
+    build_lib.build()
+    from paper_2607_13093_gb300 import sph
+    ctx = sph.Context(0)
+    w = wl.make_workload(V=n + 3000, d=K + 64, d_l=K, rows=rows, n_keep=n, seed=n, device=DEV,
+                         tau=0.9)
+    pc, ps = wl.make_payload(rows, n, seed=5, device=DEV)
+    check_endpoint(ctx, w, pc.cpu(), ps.cpu(), rows=[0, rows // 2, rows - 1])
+    ctx.close()
