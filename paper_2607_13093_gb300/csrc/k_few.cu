@@ -13,7 +13,8 @@
 //       shared memory for every tile the CTA takes
 //   A   the tile's weight rows by 16-byte cp.async with per-thread row
 //       pointers: any id pattern costs the same, and the first copies go out
-//       as soon as the ids are there.  Rows past the tile hold stale bytes
+//       as soon as the ids are there (where kernels of the same call ran
+//       before this one: before it waits for them).  Rows past the tile hold stale bytes
 //       and land in accumulator lanes that are never read.
 //   D   fp32 in TMEM, two tiles' accumulators.  Every 64 columns multiply hi,
 //       then lo, in the order of the general kernel, so z has the same bits.
@@ -64,6 +65,7 @@ struct FewParams {
   int na, KB;                // 64-column atoms of a stage, stages of a tile
   int tiles, stages, lag;    // lag: stages copied before a tile's epilogue waits
   int h16;                   // h and its rows are 16-byte aligned
+  int early;                 // ids and weights may be read before the wait (after_own)
   float* Z;                  // fused logits, row stride ldz, or nullptr
   int64_t ldz;
   const int8_t* codes;       // payload [R][n], or nullptr (none, or fused)
@@ -140,12 +142,10 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int r = row0 + 32 * i, j = tl * p.pitch + r;
-      nid[i] = (tl < p.tiles && r < p.pitch && j < p.n) ? (p.ids ? __ldg(p.ids + j) : j) : -1;
+      nid[i] = (tl < p.tiles && r < p.pitch && j < p.n) ? (p.ids ? p.ids[j] : j) : -1;
     }
   };
-  if (warp < kWorkWarps) load_ids((int)blockIdx.x);
-  else ptx::tmem_alloc(&s_tmem, kCols);
-
+  if (warp == kWorkWarps) ptx::tmem_alloc(&s_tmem, kCols);
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       ptx::mbar_init(&s_full[s], kWorkers);
@@ -159,6 +159,18 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
     ptx::mbar_init(&s_drain, 1);
     s_abort = 0;
     ptx::fence_mbar_init();
+  }
+  // As the first kernel of its call on the stream it follows the caller's
+  // work, which may be writing the ids and the weights: nothing is read, and
+  // no dependent kernel is let go, before the wait.  Behind kernels of its
+  // own call it started after the caller's work had completed (the first of
+  // them waited for that before it let anything start).
+  if (warp < kWorkWarps) {
+    if (!p.early) {
+      ptx::griddep_wait();
+      ptx::griddep_launch_dependents();
+    }
+    load_ids((int)blockIdx.x);
   }
   ptx::tc_fence_before();
   __syncthreads();
@@ -180,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
     // ---------------------------------------------------------- MMA issuer
     // (the whole warp runs the loop, one elected lane issues: see the PTX
     // wrappers)
-    ptx::griddep_launch_dependents();
+    if (p.early) ptx::griddep_launch_dependents();
     constexpr uint32_t idesc = ptx::idesc_bf16_f32(kTileIds, NR);
     int stage = 0;
     uint32_t phase = 0;
@@ -254,11 +266,11 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
       if (++lstage == S) { lstage = 0; lphase ^= 1; }
     };
     // The weights and ids come from the caller: the first stages' weights go
-    // out before the wait for the kernels before this one.
+    // out before the wait for this call's earlier kernels (whose payload the
+    // epilogue reads).
     const int ahead = min(total, p.lag + 1);
     for (int i = 0; i < ahead; ++i) copy_a();
     ptx::griddep_wait();
-    ptx::griddep_launch_dependents();
 
     // epilogue: a warp reads the TMEM lanes of its quadrant (ids quad * 32 +
     // lane of the tile) and rows erow0 .. erow0 + 15
@@ -279,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
         const int8_t* cp = p.codes + (int64_t)erow0 * p.n + j;
 #pragma unroll
         for (int q = 0; q < 16; ++q, cp += p.n)
-          if (erow0 + q < p.R) pay_c[q] = __ldg(cp);
+          if (erow0 + q < p.R) pay_c[q] = *cp;
       }
     };
 #pragma unroll
@@ -294,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
       }
     } else {
       if (threadIdx.x < p.R)
-        s_rq[threadIdx.x].s = p.codes ? __ldg(p.row_scale + threadIdx.x) : 0.f;
+        s_rq[threadIdx.x].s = p.codes ? p.row_scale[threadIdx.x] : 0.f;
     }
     // the hidden states: 8-column pieces (row, column c) of every atom, four
     // pieces a thread requested before the first is converted
@@ -309,13 +321,13 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
         const int k = atom * kAtomCols + c * 8, left = (q < pieces && r < p.R) ? p.K - k : 0;
         const float* hp = p.h + (int64_t)r * p.ld_h + k;
         if (p.h16 && left >= 8) {
-          const float4 a = __ldg(reinterpret_cast<const float4*>(hp));
-          const float4 b = __ldg(reinterpret_cast<const float4*>(hp) + 1);
+          const float4 a = *reinterpret_cast<const float4*>(hp);
+          const float4 b = *(reinterpret_cast<const float4*>(hp) + 1);
           x[u][0] = a.x; x[u][1] = a.y; x[u][2] = a.z; x[u][3] = a.w;
           x[u][4] = b.x; x[u][5] = b.y; x[u][6] = b.z; x[u][7] = b.w;
         } else {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) x[u][e] = e < left ? __ldg(hp + e) : 0.f;
+          for (int e = 0; e < 8; ++e) x[u][e] = e < left ? hp[e] : 0.f;
         }
       }
 #pragma unroll
@@ -513,6 +525,7 @@ cudaError_t launch_few(const GatherGemm& g, const FewPlan& pl, float2* seg_stats
   p.W = static_cast<const uint16_t*>(g.W); p.ld_w = g.ld_w; p.ids = g.ids;
   p.pitch = pl.pitch; p.na = pl.na; p.KB = pl.KB; p.tiles = pl.tiles;
   p.stages = pl.stages; p.lag = pl.lag;
+  p.early = g.after_own;
   p.h16 = (reinterpret_cast<uintptr_t>(g.h) & 15) == 0 && g.ld_h % 4 == 0;
   p.Z = g.Y; p.ldz = g.ldy ? g.ldy : g.n;
   p.codes = g.codes; p.row_scale = g.row_scale; p.inv_tau = g.inv_tau;

@@ -1152,6 +1152,7 @@ sph_status sph_split_step(sph_ctx* ctx, const float* h, int64_t rows, int64_t ld
     gg.W = W_l; gg.ld_w = ld_wl; gg.V = V; gg.w_dtype = sph::W_BF16; gg.K = (int)d_l;
     gg.ids = keep_ids; gg.n = (int)n_keep;
     gg.Y = Z;
+    gg.after_own = true;
     if (fuse_q) {
       gg.epilogue = sph::EPI_FUSED;
       gg.yc = Y; gg.rowmax_in = rowmax; gg.codes_out = codes; gg.scale_out = scales;
@@ -1229,6 +1230,8 @@ sph_status sph_split_step(sph_ctx* ctx, const float* h, int64_t rows, int64_t ld
     gg.Y = Z + j0; gg.ldy = n_keep;
     gg.status = ctx->status; gg.finish_wait = ctx->tc_finish_wait;
     gg.inv_tau = inv_tau; gg.no_stats = true;
+    // (chunk 0 on a stream of its own follows whatever the caller put there)
+    gg.after_own = serial || q > 0;
     sph::FewPlan few{};
     if (few_route(ctx, gg, sm_end, &few)) {
       st = launch_status(ctx, sph::launch_few(gg, few, nullptr, ctx->spin_limit, es),

@@ -31,7 +31,13 @@ extern thread_local long long launch_count;
 // Launch with programmatic stream serialization: the kernel may start while
 // the previous kernel of the stream is still running, and must call
 // griddepcontrol.wait (ptx::griddep_wait) before it touches memory that an
-// earlier kernel writes or reads.  Every kernel of this library does so.
+// earlier kernel writes or reads.  Every kernel of this library does so.  The
+// earlier kernel may be the caller's, which writes anything the call is given,
+// ids and weights too, and may let its dependents start early itself: the
+// first kernel that an API call launches on a stream waits before it reads
+// anything and before it lets its own dependents start.  The later ones of
+// the call start only after that wait, so they may read the caller's ids and
+// weights (not what kernels of the call write) before their own.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                        cudaStream_t st, Args&&... args) {
@@ -105,6 +111,7 @@ struct GatherGemm {
   unsigned* status;        // device error word
   long long finish_wait = 1ll << 15;   // split-tile finisher poll (cycles; 0: none)
   bool no_stats = false;   // endpoint: skip the softmax statistics (Gumbel-max draw)
+  bool after_own = false;  // the kernel before it on its stream is of the same API call
   // cloud GEMV in one launch: the last block to arrive (q_ticket, which it
   // resets) quantizes every row (Eq. 18) into q_codes / q_scale and clears
   // the row maxima for the next call; nullptr: the quantize pass does it
