@@ -26,7 +26,7 @@ constexpr int kQThreads = 256;
 constexpr int kQSpan = kQThreads * kQVec;
 
 __global__ void __launch_bounds__(kQThreads)
-quantize_kernel(const float* __restrict__ Y, const unsigned* __restrict__ rowmax, int rows,
+quantize_kernel(const float* Y, const unsigned* rowmax, int rows,
                 int n, int8_t* __restrict__ codes, float* __restrict__ row_scale) {
   ptx::griddep_wait();
   ptx::griddep_launch_dependents();

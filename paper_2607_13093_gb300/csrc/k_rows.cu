@@ -55,7 +55,7 @@ __device__ __forceinline__ float seg_weight(float2 st, float M, float inv_tau) {
 // 22.5 us on the spec workload's 66 MB).
 constexpr int kSegRow = 36;             // words per segment in the tile
 __global__ void __launch_bounds__(kWarps * 32)
-seg_stats_kernel(const float* __restrict__ Z, int rows, int n, int nseg, int nchunk,
+seg_stats_kernel(const float* Z, int rows, int n, int nseg, int nchunk,
                  float inv_tau, float2* __restrict__ stats, float2* __restrict__ cstats) {
   __shared__ __align__(16) float tile[kWarps][kSeg * kSegRow];
   ptx::griddep_wait();
@@ -133,7 +133,7 @@ seg_stats_kernel(const float* __restrict__ Z, int rows, int n, int nseg, int nch
 // Chunk statistics from segment statistics (rows of `nseg` entries): a warp
 // per chunk.
 __global__ void __launch_bounds__(kWarps * 32)
-chunk_stats_kernel(const float2* __restrict__ stats, int rows, int nseg, int nchunk,
+chunk_stats_kernel(const float2* stats, int rows, int nseg, int nchunk,
                    float inv_tau, float2* __restrict__ cstats) {
   ptx::griddep_wait();
   ptx::griddep_launch_dependents();
@@ -309,7 +309,7 @@ struct ZRowRecomputed {
     for (; k + 8 <= K; k += 8) dot8(__ldg(reinterpret_cast<const uint4*>(w + k)), k, a);
     for (; k < K; ++k) a[0] = fmaf(__ldg(h + k), __uint_as_float((unsigned)w[k] << 16), a[0]);
     const float z = (a[0] + a[1]) + (a[2] + a[3]);
-    return c ? fmaf((float)__ldg(c + j), s, z) : z;
+    return c ? fmaf((float)c[j], s, z) : z;
   }
   // The same z by the whole warp (every lane gets it): lane l takes the
   // 8-element pieces l, l + 32, ... of the row, then a warp sum.
@@ -322,7 +322,7 @@ struct ZRowRecomputed {
     for (int k = K8 + lane; k < K; k += 32)
       a[0] = fmaf(__ldg(h + k), __uint_as_float((unsigned)w[k] << 16), a[0]);
     const float z = warp_sum((a[0] + a[1]) + (a[2] + a[3]));
-    return c ? fmaf((float)__ldg(c + j), s, z) : z;
+    return c ? fmaf((float)c[j], s, z) : z;
   }
 };
 struct ZRowsStored {
@@ -339,7 +339,7 @@ struct ZRowsRecomputed {
     const float* hr = zs.h + r * zs.ld_h;
     return ZRowRecomputed{hr, zs.K, static_cast<const uint16_t*>(zs.W), zs.ld_w,
                           zs.ids, zs.codes ? zs.codes + r * n : nullptr,
-                          zs.codes ? __ldg(zs.row_scale + r) : 0.f,
+                          zs.codes ? zs.row_scale[r] : 0.f,
                           (reinterpret_cast<uintptr_t>(hr) & 15) == 0};
   }
 };
@@ -386,8 +386,8 @@ __device__ __forceinline__ float stats_max(const float2* cst, int nchunk, int la
 template <class ZRows>
 __global__ void __launch_bounds__(kWarps * 32)
 sample_seg_kernel(const ZRows zr, int rows, int n,
-                  const float2* __restrict__ stats, int nseg,
-                  const float2* __restrict__ cstats, const int32_t* __restrict__ ids,
+                  const float2* stats, int nseg,
+                  const float2* cstats, const int32_t* ids,
                   float inv_tau, uint64_t seed, uint64_t offset,
                   int32_t* __restrict__ tokens) {
   ptx::griddep_wait();
@@ -417,8 +417,8 @@ constexpr int kMaxFusedChunks = 4096;   // shared memory: 8 bytes per chunk
 constexpr int kFusedU = 4;              // chunks in flight per warp
 template <class ZRows>
 __global__ void __launch_bounds__(1024)
-sample_rows_kernel(const ZRows zr, int n, const float2* __restrict__ stats,
-                   int nseg, const int32_t* __restrict__ ids, float inv_tau, uint64_t seed,
+sample_rows_kernel(const ZRows zr, int n, const float2* stats,
+                   int nseg, const int32_t* ids, float inv_tau, uint64_t seed,
                    uint64_t offset, int32_t* __restrict__ tokens) {
   extern __shared__ float2 s_cst[];
   ptx::griddep_wait();
@@ -528,7 +528,7 @@ __device__ __forceinline__ int warp_argmax(const ZR& z, int n, const float2* st,
 // tile tb; this lane's segment's (max, sum of exp), the same tree of sums.
 // (The pass itself keeps its own text: with this function called from its
 // loop, 3 rows x 32000 ids took 18.98 us instead of 18.38.)
-__device__ __forceinline__ float2 chunk_segment_stats(const float* __restrict__ z, int left,
+__device__ __forceinline__ float2 chunk_segment_stats(const float* z, int left,
                                                       float* tb, float l2t, int lane) {
   if (left >= kSeg * kSeg && ((reinterpret_cast<uintptr_t>(z) & 15) == 0)) {
 #pragma unroll
@@ -585,7 +585,7 @@ __device__ __forceinline__ float2 chunk_segment_stats(const float* __restrict__ 
 constexpr int kShortChunks = kWarps;
 constexpr int kShortRows = 16;
 __global__ void __launch_bounds__(kWarps * 32)
-sample_short_kernel(const ZRowsStored zr, int n, const int32_t* __restrict__ ids, float inv_tau,
+sample_short_kernel(const ZRowsStored zr, int n, const int32_t* ids, float inv_tau,
                     uint64_t seed, uint64_t offset, int greedy, int32_t* __restrict__ tokens) {
   __shared__ __align__(16) float tile[kWarps][kSeg * kSegRow];
   __shared__ float2 s_seg[kShortChunks * kSeg];
@@ -630,7 +630,7 @@ sample_short_kernel(const ZRowsStored zr, int n, const int32_t* __restrict__ ids
 constexpr uint32_t kGumbelTag = 0x80000000u;
 constexpr int kGumbelThreads = 256;
 __global__ void __launch_bounds__(kGumbelThreads)
-gumbel_rows_kernel(const float* __restrict__ Z, int n, const int32_t* __restrict__ ids,
+gumbel_rows_kernel(const float* Z, int n, const int32_t* ids,
                    float inv_tau, uint64_t seed, uint64_t offset,
                    int32_t* __restrict__ tokens) {
   __shared__ float s_key[kGumbelThreads / 32];
@@ -690,8 +690,8 @@ gumbel_rows_kernel(const float* __restrict__ Z, int n, const int32_t* __restrict
 // One warp per row: vocabulary ids into tokens and/or compact indices.
 template <class ZRows>
 __global__ void __launch_bounds__(kWarps * 32)
-greedy_kernel(const ZRows zr, int rows, int n, const float2* __restrict__ stats,
-              int nseg, const int32_t* __restrict__ ids, int32_t* __restrict__ tokens,
+greedy_kernel(const ZRows zr, int rows, int n, const float2* stats,
+              int nseg, const int32_t* ids, int32_t* __restrict__ tokens,
               int32_t* __restrict__ compact) {
   ptx::griddep_wait();
   ptx::griddep_launch_dependents();
@@ -752,10 +752,10 @@ __device__ __forceinline__ int first_rejection(const int32_t* acc, int s, int k,
 // One warp per target row: the row's softmax maximum and normaliser and,
 // for a draft position, the acceptance test r_i * q_i(x_i) < p_i(x_i).
 __global__ void __launch_bounds__(kWarps * 32)
-verify_rows_kernel(const float* __restrict__ Z, const float2* __restrict__ cstats,
-                   int nchunk, int n, int sessions, int k, const int32_t* __restrict__ ids,
-                   int V, float inv_tau, const int32_t* __restrict__ draft,
-                   const float* __restrict__ q, uint64_t seed, uint64_t offset,
+verify_rows_kernel(const float* Z, const float2* cstats,
+                   int nchunk, int n, int sessions, int k, const int32_t* ids,
+                   int V, float inv_tau, const int32_t* draft,
+                   const float* q, uint64_t seed, uint64_t offset,
                    float2* __restrict__ rowMS, int32_t* __restrict__ acc,
                    int32_t* __restrict__ xis) {
   ptx::griddep_wait();
@@ -795,10 +795,10 @@ verify_rows_kernel(const float* __restrict__ Z, const float2* __restrict__ cstat
 // Segment and chunk weights of the residual distribution at each session's
 // first rejection: a warp per (session, chunk).
 __global__ void __launch_bounds__(kWarps * 32)
-verify_residual_kernel(const float* __restrict__ Z, int n, int nseg, int nchunk,
-                       int sessions, int k, const float* __restrict__ q, float inv_tau,
-                       const float2* __restrict__ rowMS, const int32_t* __restrict__ acc,
-                       const int32_t* __restrict__ xis, float* __restrict__ resw,
+verify_residual_kernel(const float* Z, int n, int nseg, int nchunk,
+                       int sessions, int k, const float* q, float inv_tau,
+                       const float2* rowMS, const int32_t* acc,
+                       const int32_t* xis, float* __restrict__ resw,
                        float* __restrict__ resc) {
   ptx::griddep_wait();
   ptx::griddep_launch_dependents();
@@ -849,9 +849,9 @@ verify_residual_kernel(const float* __restrict__ Z, int n, int nseg, int nchunk,
 // Greedy verification, one thread per session: accept while the draft is
 // the target's argmax; the next token is the argmax at the first mismatch,
 // or at the bonus position.
-__global__ void greedy_verify_kernel(const int32_t* __restrict__ amax, int sessions, int k,
-                                     int n, const int32_t* __restrict__ ids, int V,
-                                     const int32_t* __restrict__ draft,
+__global__ void greedy_verify_kernel(const int32_t* amax, int sessions, int k,
+                                     int n, const int32_t* ids, int V,
+                                     const int32_t* draft,
                                      int32_t* __restrict__ n_acc,
                                      int32_t* __restrict__ next_token) {
   ptx::griddep_wait();
@@ -868,13 +868,13 @@ __global__ void greedy_verify_kernel(const int32_t* __restrict__ amax, int sessi
 // One warp per session: the draw, from the residual (or, if that is all
 // zero, from p_i) at the first rejection, else the bonus draw from p_k.
 __global__ void __launch_bounds__(kWarps * 32)
-verify_draw_kernel(const float* __restrict__ Z, int n, const float2* __restrict__ stats,
-                   const float2* __restrict__ cstats, int nseg, int nchunk, int sessions,
-                   int k, const int32_t* __restrict__ ids, const float* __restrict__ q,
+verify_draw_kernel(const float* Z, int n, const float2* stats,
+                   const float2* cstats, int nseg, int nchunk, int sessions,
+                   int k, const int32_t* ids, const float* q,
                    float inv_tau, uint64_t seed, uint64_t offset,
-                   const float2* __restrict__ rowMS, const int32_t* __restrict__ acc,
-                   const int32_t* __restrict__ xis, const float* __restrict__ resw,
-                   const float* __restrict__ resc, int32_t* __restrict__ n_acc,
+                   const float2* rowMS, const int32_t* acc,
+                   const int32_t* xis, const float* resw,
+                   const float* resc, int32_t* __restrict__ n_acc,
                    int32_t* __restrict__ next_token) {
   ptx::griddep_wait();
   ptx::griddep_launch_dependents();

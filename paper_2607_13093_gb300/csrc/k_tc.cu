@@ -261,7 +261,7 @@ __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)
       float y[16];
       if (p.h_scale) {
 #pragma unroll
-        for (int q = 0; q < 16; ++q) y[q] = (v[q] * __ldg(p.h_scale + row0 + q)) * ws + b;
+        for (int q = 0; q < 16; ++q) y[q] = (v[q] * p.h_scale[row0 + q]) * ws + b;
       } else {
 #pragma unroll
         for (int q = 0; q < 16; ++q) y[q] = v[q] * ws + b;
@@ -285,7 +285,7 @@ __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)
       const int r = row0 + q;
       m[q] = 0.f;
       if (vj && r < p.R) {
-        const float y = (p.h_scale ? v[q] * __ldg(p.h_scale + r) : v[q]) * ws + b;
+        const float y = (p.h_scale ? v[q] * p.h_scale[r] : v[q]) * ws + b;
         const int64_t o = (int64_t)r * p.n + j;
         if (p.partial_out) p.partial_out[o] = y;
         const float yc = fminf(fmaxf(y, -p.clip), p.clip);
@@ -1425,7 +1425,7 @@ __device__ __forceinline__ void split_group(const float (&x)[8], int hilo, uint4
 
 constexpr int kSplitThreads = 128;
 __global__ void __launch_bounds__(kSplitThreads, 16)
-split_h_kernel(const float* __restrict__ h, int64_t ld_h, int R, int K, int Rp, int Kp,
+split_h_kernel(const float* h, int64_t ld_h, int R, int K, int Rp, int Kp,
                int hilo, __nv_bfloat16* __restrict__ Hs, int* __restrict__ counters,
                int ncounters, unsigned* __restrict__ rowmax) {
   ptx::griddep_wait();
@@ -1444,13 +1444,13 @@ split_h_kernel(const float* __restrict__ h, int64_t ld_h, int R, int K, int Rp, 
     float x[8];
     const float* src = h + (int64_t)r * ld_h + c0;
     if (r < R && vec && c0 + 8 <= K) {
-      const float4 a = __ldg(reinterpret_cast<const float4*>(src));
-      const float4 b = __ldg(reinterpret_cast<const float4*>(src) + 1);
+      const float4 a = *reinterpret_cast<const float4*>(src);
+      const float4 b = *(reinterpret_cast<const float4*>(src) + 1);
       x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
       x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
     } else {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = (r < R && c0 + i < K) ? __ldg(src + i) : 0.f;
+      for (int i = 0; i < 8; ++i) x[i] = (r < R && c0 + i < K) ? src[i] : 0.f;
     }
     uint4 hi, lo;
     split_group(x, hilo, &hi, &lo);
@@ -1471,7 +1471,7 @@ split_h_kernel(const float* __restrict__ h, int64_t ld_h, int R, int K, int Rp, 
 // two 4-bit halves.  Also clears the split-tile counters and row maxima.
 constexpr int kSplit8Threads = 256;
 __global__ void __launch_bounds__(kSplit8Threads)
-split_h_e4m3_kernel(const float* __restrict__ h, int64_t ld_h, int R, int K, int Rp, int Kp,
+split_h_e4m3_kernel(const float* h, int64_t ld_h, int R, int K, int Rp, int Kp,
                     int planes, uint8_t* __restrict__ Hs, float* __restrict__ h_scale,
                     int* __restrict__ counters, int ncounters, unsigned* __restrict__ rowmax,
                     int act_bf16) {
@@ -1486,7 +1486,7 @@ split_h_e4m3_kernel(const float* __restrict__ h, int64_t ld_h, int R, int K, int
   const int r = blockIdx.x;
   const float* hr = h + (int64_t)r * ld_h;
   auto value = [&](int c) {
-    float x = (r < R && c < K) ? __ldg(hr + c) : 0.f;
+    float x = (r < R && c < K) ? hr[c] : 0.f;
     if (act_bf16) x = __bfloat162float(__float2bfloat16_rn(x));
     return x;
   };
@@ -1495,7 +1495,7 @@ split_h_e4m3_kernel(const float* __restrict__ h, int64_t ld_h, int R, int K, int
   const bool v16 = (reinterpret_cast<uintptr_t>(hr) & 15) == 0;
   auto value4 = [&](int c, float (&x)[4]) {
     if (v16 && r < R && c + 4 <= K) {
-      const float4 t = __ldg(reinterpret_cast<const float4*>(hr + c));
+      const float4 t = *reinterpret_cast<const float4*>(hr + c);
       x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
       if (act_bf16) {
 #pragma unroll

@@ -38,6 +38,11 @@ extern thread_local long long launch_count;
 // anything and before it lets its own dependents start.  The later ones of
 // the call start only after that wait, so they may read the caller's ids and
 // weights (not what kernels of the call write) before their own.
+// What is read behind the wait is read with coherent loads: a non-coherent one
+// (__ldg, or a const __restrict__ parameter) is free to move before it, and is
+// only for memory whose writer had finished before the kernel could start --
+// for the kernels that follow an operand split or a statistics pass of their
+// own call, what the call was given or wrote before that pass.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                        cudaStream_t st, Args&&... args) {

@@ -1,5 +1,5 @@
-"""A call reads what it is given -- ids and weights as well -- only after the
-caller's kernel before it in the stream has written it, also where that kernel
+"""A call reads what it is given -- ids and weights as well as hidden states and
+payload -- only after the caller's kernel before it in the stream has written it, also where that kernel
 lets its dependents start early (programmatic dependent launch), as kernels of
 other libraries do.  The writer here does so and writes 50 us later; both the
 old and the new contents are valid, so a call that did not wait would answer
@@ -62,18 +62,20 @@ def ctx():
 # rows: the GEMV, the few-row endpoint kernel, the general tensor-core kernel
 # on single CTAs and on pairs
 @pytest.mark.parametrize("rows", [2, 16, 48, 256])
-@pytest.mark.parametrize("late", ["keep_ids", "weights"])
+@pytest.mark.parametrize("late", ["keep_ids", "weights", "full", "hidden", "payload"])
 @pytest.mark.parametrize("call", ["cloud", "endpoint", "logits", "step", "streamed", "serial",
                                   "verify"])
 def test_call_reads_after_the_callers_kernel(ctx, writer, call, late, rows):
-    if call == "verify" and late == "weights":
-        pytest.skip("verification takes no weights")
-    V, n, k = 6000, 3000, 1
+    if (call == "verify" and late != "keep_ids") or (
+            late == "payload" and call not in ("endpoint", "logits")):
+        pytest.skip("the call takes no such input")
+    # ("full": the weights of a call over the whole vocabulary, without ids)
+    V, n, k = 3000 if late == "full" else 6000, 3000, 1
     w = wl.make_workload(V=V, d=640, d_l=128, rows=rows, n_keep=n, seed=71, device=DEV, k=k,
                          sessions=rows // (k + 1))
     pc, ps = wl.make_payload(rows, n, seed=3, device=DEV)
     zt = torch.randn(rows, n, device=DEV)
-    ids = w.keep_ids.clone()
+    ids = None if late == "full" else w.keep_ids.clone()
     old_ids = torch.arange(n, dtype=torch.int32, device=DEV)
     codes, tok = (torch.empty(s, dtype=t, device=DEV)
                   for s, t in ((rows * n, torch.int8), (rows, torch.int32)))
@@ -110,19 +112,19 @@ def test_call_reads_after_the_callers_kernel(ctx, writer, call, late, rows):
         torch.cuda.synchronize()
         return out
 
-    # the weights (one row further on before the write) of the call's last
-    # contraction; streamed: written on the endpoint's own stream, which the
-    # call's endpoint half follows
+    # the weights are those of the call's last contraction (streamed: written on
+    # the endpoint's own stream, which the call's endpoint half follows)
     if late == "keep_ids":
         dst, new, old = ids, w.keep_ids, old_ids
     else:
-        dst = w.W_h if call == "cloud" else w.W_l
+        # before the write: one row further on
+        dst = {"payload": pc, "hidden": w.h}.get(late, w.W_h if call == "cloud" else w.W_l)
         new, old = dst.clone(), dst.roll(1, 0).contiguous()
     want = snapshot()
     dst.copy_(old)
     was = snapshot()
     assert any(not torch.equal(a, b) for a, b in zip(want, was))
-    on_es = call == "streamed" and late == "weights"
+    on_es = call == "streamed" and late in ("weights", "full")
     for _ in range(3):
         dst.copy_(old)
         torch.cuda.synchronize()
