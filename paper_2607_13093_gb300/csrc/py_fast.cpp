@@ -44,11 +44,17 @@ struct Args {
     else if (d != dev) { ok = false; return nullptr; }
     return &t;
   }
-  // a 2-D operand with unit inner stride
-  const at::Tensor* matrix(int i) {
+  // a 2-D operand with unit inner stride, and its address and row stride
+  struct Matrix {
+    const at::Tensor* t = nullptr;
+    const void* p = nullptr;
+    long long ld = 0;
+    const at::Tensor* operator->() const { return t; }
+  };
+  Matrix matrix(int i) {
     const at::Tensor* t = tensor(i);
-    if (t && (t->dim() != 2 || t->stride(1) != 1)) { ok = false; return nullptr; }
-    return t;
+    if (!t || t->dim() != 2 || t->stride(1) != 1) { ok = false; return {}; }
+    return {t, t->const_data_ptr(), (long long)t->stride(0)};
   }
   // a dense buffer of `type` with at least `count` elements (None: nullptr)
   template <class T>
@@ -84,8 +90,8 @@ struct Args {
     return 0.f;
   }
   // bf16 or e4m3 weights
-  sph_dtype weights(const at::Tensor* w) {
-    if (!w) { ok = false; return SPH_DTYPE_BF16; }
+  sph_dtype weights(const Matrix& w) {
+    if (!w.t) { ok = false; return SPH_DTYPE_BF16; }
     if (w->scalar_type() == c10::kBFloat16) return SPH_DTYPE_BF16;
     if (w->scalar_type() == c10::kFloat8_e4m3fn) return SPH_DTYPE_FP8_E4M3;
     ok = false;
@@ -98,18 +104,21 @@ PyObject* outcome(sph_status st, size_t bytes) {
   return PyLong_FromLongLong(st == SPH_OK ? (long long)bytes : -1 - (long long)st);
 }
 
-// The library call without the interpreter lock (as ctypes makes it).
+// The interpreter lock released for the library call (as ctypes makes it),
+// and held again however that ends.  Everything a tensor is asked for, which
+// may throw, is asked before.
+struct Unlocked {
+  PyThreadState* saved = PyEval_SaveThread();
+  ~Unlocked() { PyEval_RestoreThread(saved); }
+};
 template <class F>
 sph_status unlocked(F&& f) {
-  sph_status st;
-  Py_BEGIN_ALLOW_THREADS
-  st = f();
-  Py_END_ALLOW_THREADS
-  return st;
+  Unlocked u;
+  return f();
 }
 
 // No C++ exception crosses into the interpreter: whatever a tensor refuses
-// to say is left to the Python path.
+// to say (one without storage has no address) is left to the Python path.
 template <class F>
 PyObject* guarded(F&& f) {
   try {
@@ -127,8 +136,8 @@ PyObject* partial_logits(PyObject*, PyObject* const* argv, Py_ssize_t n) {
     if (n != 11) return not_taken();
     Args A{argv};
     auto* ctx = reinterpret_cast<sph_ctx*>((uintptr_t)A.word(0));
-    const at::Tensor* h = A.matrix(1);
-    const at::Tensor* W = A.matrix(2);
+    const Args::Matrix h = A.matrix(1);
+    const Args::Matrix W = A.matrix(2);
     if (!A.ok || h->scalar_type() != c10::kFloat) return not_taken();
     const sph_dtype wdt = A.weights(W);
     const long long R = h->size(0), dh = h->size(1), V = W->size(0);
@@ -145,9 +154,8 @@ PyObject* partial_logits(PyObject*, PyObject* const* argv, Py_ssize_t n) {
     if (!A.ok || !ctx) return not_taken();
     size_t pb = 0;
     const sph_status st = unlocked([&] {
-      return p_partial(ctx, h->const_data_ptr<float>(), R, h->stride(0), W->const_data_ptr(), wdt,
-                       V, dh, W->stride(0), ws, bias, keep, nk, clip, (sph_act_mode)act, codes,
-                       scale, part, &pb);
+      return p_partial(ctx, static_cast<const float*>(h.p), R, h.ld, W.p, wdt, V, dh, W.ld, ws,
+                       bias, keep, nk, clip, (sph_act_mode)act, codes, scale, part, &pb);
     });
     return outcome(st, pb);
   });
@@ -160,8 +168,8 @@ PyObject* fuse_sample(PyObject*, PyObject* const* argv, Py_ssize_t n) {
     if (n != 11) return not_taken();
     Args A{argv};
     auto* ctx = reinterpret_cast<sph_ctx*>((uintptr_t)A.word(0));
-    const at::Tensor* h = A.matrix(3);
-    const at::Tensor* W = A.matrix(4);
+    const Args::Matrix h = A.matrix(3);
+    const Args::Matrix W = A.matrix(4);
     if (!A.ok || h->scalar_type() != c10::kFloat || W->scalar_type() != c10::kBFloat16)
       return not_taken();
     const long long R = h->size(0), dl = h->size(1), V = W->size(0);
@@ -176,9 +184,8 @@ PyObject* fuse_sample(PyObject*, PyObject* const* argv, Py_ssize_t n) {
     float* z = A.dense<float>(10, c10::kFloat, R * nk);
     if (!A.ok || !ctx) return not_taken();
     return outcome(unlocked([&] {
-      return p_fuse(ctx, codes, scale, R, h->const_data_ptr<float>(), h->stride(0),
-                    W->const_data_ptr(), V, dl, W->stride(0), keep, nk, tau, seed, offset, tokens,
-                    z);
+      return p_fuse(ctx, codes, scale, R, static_cast<const float*>(h.p), h.ld, W.p, V, dl, W.ld,
+                    keep, nk, tau, seed, offset, tokens, z);
     }), 0);
   });
 }
@@ -190,10 +197,10 @@ PyObject* split_step(PyObject*, PyObject* const* argv, Py_ssize_t n) {
     if (n != 18) return not_taken();
     Args A{argv};
     auto* ctx = reinterpret_cast<sph_ctx*>((uintptr_t)A.word(0));
-    const at::Tensor* h = A.matrix(1);
+    const Args::Matrix h = A.matrix(1);
     const long long dl = A.integer(2);
-    const at::Tensor* Wh = A.matrix(3);
-    const at::Tensor* Wl = A.matrix(4);
+    const Args::Matrix Wh = A.matrix(3);
+    const Args::Matrix Wl = A.matrix(4);
     if (!A.ok || h->scalar_type() != c10::kFloat || Wl->scalar_type() != c10::kBFloat16)
       return not_taken();
     const sph_dtype wdt = A.weights(Wh);
@@ -217,9 +224,8 @@ PyObject* split_step(PyObject*, PyObject* const* argv, Py_ssize_t n) {
     if (!A.ok || !ctx) return not_taken();
     size_t pb = 0;
     const sph_status st = unlocked([&] {
-      return p_split(ctx, h->const_data_ptr<float>(), R, h->stride(0), dl, dh,
-                     Wh->const_data_ptr(), wdt, ws, Wh->stride(0), Wl->const_data_ptr(),
-                     Wl->stride(0), V, bias, keep, nk, clip, (sph_act_mode)act, tau, seed, offset,
+      return p_split(ctx, static_cast<const float*>(h.p), R, h.ld, dl, dh, Wh.p, wdt, ws, Wh.ld,
+                     Wl.p, Wl.ld, V, bias, keep, nk, clip, (sph_act_mode)act, tau, seed, offset,
                      chunk, es, codes, scales, tokens, nullptr, &pb);
     });
     return outcome(st, pb);

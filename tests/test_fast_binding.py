@@ -1,5 +1,9 @@
 """The native argument marshalling (csrc/py_fast.cpp) takes plain calls and
 leaves the rest to the Python checks: same results either way, same errors."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -38,6 +42,42 @@ def test_anything_not_plain_is_left_to_python(sph):
         sph.sph_partial_logits(None, h, W, codes=codes, row_scale=scale)
     with pytest.raises(ValueError, match="CUDA tensor"):
         sph.sph_verify_draft(None, h, 1, 1, tok, n_accepted=tok, next_token=tok)
+
+
+NO_STORAGE = """
+import sys
+import torch
+from torch._subclasses.fake_tensor import FakeTensorMode
+from paper_2607_13093_gb300 import sph
+
+f, got, bf = sph._fast, [], torch.bfloat16
+
+def call(h):          # plain CUDA tensors by type, device and shape, without storage
+    W, n = h.to(bf), h.to(torch.int32)
+    assert type(h) is torch.Tensor and h.is_cuda
+    got.append({
+        "partial": lambda: f.partial_logits(1, h, W, None, 30.0, None, None, 0, None, None, None),
+        "fuse": lambda: f.fuse_sample(1, None, None, h, W, None, 1.0, 1, 2, None, None),
+        "split": lambda: f.split_step(1, h, 8, W, W, None, 30.0, None, None, 0, 1.0, 1, 2, 0, 0,
+                                      None, None, None),
+        "verify": lambda: f.verify_draft(1, h, 1, 1, n, None, None, 1.0, 1, 2, n, n),
+    }[sys.argv[1]]())
+    return h
+
+with FakeTensorMode():
+    torch.vmap(call)(torch.empty(3, 2, 16, device="cuda"))
+assert got == [sph._NOT_TAKEN], got
+"""
+
+
+@pytest.mark.parametrize("call", ["partial", "fuse", "split", "verify"])
+def test_a_tensor_without_storage_is_left_to_python(sph, call):
+    # (a process of its own: asking such a tensor for its address throws, and
+    # an exception without the interpreter lock ends the interpreter)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", NO_STORAGE, call], cwd=root, capture_output=True,
+                       text=True)
+    assert r.returncode == 0, r.stderr
 
 
 @pytest.mark.gpu
