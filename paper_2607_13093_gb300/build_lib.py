@@ -3,9 +3,11 @@
 Each translation unit compiles in parallel to an object file under _lib/;
 the objects link into _lib/libsph.so against the shared CUDA runtime (the
 same libcudart the process already uses for PyTorch).  A source newer than
-its object, or a changed header, triggers a rebuild of that unit.  Beside it
-g++ builds _lib/py_fast.so, the binding's native argument marshalling,
-against the installed PyTorch.
+its object, or a changed header, triggers a rebuild of that unit.  The library
+needs nvcc alone.  Where PyTorch is installed, nvcc's host compiler builds the
+binding's native argument marshalling beside it, in a file that carries the
+PyTorch and Python it was built against in its name (fast_path): another
+PyTorch or Python never loads it.
 """
 from __future__ import annotations
 
@@ -22,7 +24,6 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OUT = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUT, "libsph.so")
-FAST = os.path.join(OUT, "py_fast.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
@@ -54,20 +55,32 @@ def _stale(obj: str, src: str, newest_header: float) -> bool:
     return os.path.getmtime(src) > t or newest_header > t
 
 
-def _fast_cmd(src: str):
+def fast_path():
+    """File of the native argument marshalling for the running Python and the
+    installed PyTorch; None without PyTorch."""
+    try:
+        import torch
+    except ImportError:
+        return None
+    abi = sysconfig.get_config_var("SOABI")
+    return os.path.join(OUT, f"py_fast.{abi}.torch-{torch.__version__}.so")
+
+
+def _fast_cmd(cc: str, src: str, out: str):
     import torch
     root = os.path.dirname(os.path.abspath(torch.__file__))
     inc, lib = os.path.join(root, "include"), os.path.join(root, "lib")
     abi = int(getattr(torch._C, "_GLIBCXX_USE_CXX11_ABI", True))
-    return [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-fPIC", "-shared",
+    return [cc, "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-shared", "-cudart", "none",
             f"-D_GLIBCXX_USE_CXX11_ABI={abi}", "-I", INCLUDE,
             "-I", sysconfig.get_paths()["include"], "-I", inc,
-            "-I", os.path.join(inc, "torch", "csrc", "api", "include"), src, "-o", FAST,
-            "-L", lib, f"-Wl,-rpath,{lib}", "-lc10", "-ltorch_cpu", "-ltorch_python", "-ldl"]
+            "-I", os.path.join(inc, "torch", "csrc", "api", "include"), src, "-o", out,
+            "-L", lib, "-Xlinker", f"-rpath={lib}", "-lc10", "-ltorch_cpu", "-ltorch_python", "-ldl"]
 
 
 def build(verbose: bool = False, force: bool = False, extra_flags=()) -> str:
-    """Compile every csrc/*.cu and link _lib/libsph.so; returns its path."""
+    """Compile every csrc/*.cu and link _lib/libsph.so, and build the native
+    marshalling where PyTorch is installed; returns the library's path."""
     os.makedirs(OUT, exist_ok=True)
     cc = nvcc()
     srcs = _sources()
@@ -83,9 +96,10 @@ def build(verbose: bool = False, force: bool = False, extra_flags=()) -> str:
             jobs.append((s, cmd))
 
     relink = bool(jobs) or force or not os.path.exists(LIB)
-    fast_src = os.path.join(CSRC, "py_fast.cpp")
-    if force or _stale(FAST, fast_src, newest_header):
-        jobs.append((fast_src, _fast_cmd(fast_src)))
+    fast, fast_src = fast_path(), os.path.join(CSRC, "py_fast.cpp")
+    newest = max(newest_header, os.path.getmtime(os.path.abspath(__file__)))
+    if fast and (force or _stale(fast, fast_src, newest)):
+        jobs.append((fast_src, _fast_cmd(cc, fast_src, fast)))
 
     def run(job):
         src, cmd = job
@@ -101,16 +115,16 @@ def build(verbose: bool = False, force: bool = False, extra_flags=()) -> str:
                 print(r.stdout + r.stderr, flush=True)
             if r.returncode != 0:
                 failed.append((src, r.stdout + r.stderr))
-    if failed:
-        msg = "\n".join(f"{s}:\n{out}" for s, out in failed)
-        raise RuntimeError("compiling failed:\n" + msg)
-    if relink:
+    if relink and not any(s != fast_src for s, _ in failed):
         cmd = [cc, *ARCH, "-shared", "-cudart", "shared", "-o", LIB, *objs]
         if verbose:
             print(" ".join(cmd), flush=True)
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("link failed:\n" + r.stdout + r.stderr)
+    if failed:          # (the marshalling's failure leaves the library linked)
+        msg = "\n".join(f"{s}:\n{out}" for s, out in failed)
+        raise RuntimeError("compiling failed:\n" + msg)
     return LIB
 
 

@@ -132,10 +132,11 @@ LIB_PATH = _LIB_PATH
 
 def _load_fast():
     import importlib.util
-    path = os.path.join(os.path.dirname(_LIB_PATH), "py_fast.so")
-    if not os.path.exists(path):
+    from .build_lib import fast_path
+    path = fast_path()
+    if path is None or not os.path.exists(path):
         raise RuntimeError(
-            f"py_fast.so is not built ({path}); run "
+            f"the native marshalling is not built for this PyTorch and Python ({path}); run "
             "`python -c 'import __graft_entry__ as g; g.build()'` first")
     spec = importlib.util.spec_from_file_location("py_fast", path)
     mod = importlib.util.module_from_spec(spec)
