@@ -204,6 +204,16 @@ typedef enum sph_option {
                                small buffer of the context that the call
                                leaves cleared); 1 always a separate quantize
                                pass.  Bit-identical codes and scales.      */
+  SPH_OPT_FEW_ROWS = 15,    /* the endpoint contraction's few-row kernel:
+                               0 automatic (default: for 4..32 rows, from
+                               SPH_OPT_TC_MIN_ROWS on, over d_l <= 512, where
+                               the general tensor-core kernel would take
+                               whole tiles too), 1 never.  The options that
+                               shape the general kernel ask for it as well:
+                               any SPH_OPT_TC_SCHEDULE, _STAGES, _BLOCK_K,
+                               _MAX_BN or _TILE_M but 0, SPH_OPT_TC_PAIR = 1
+                               and SPH_OPT_ENDPOINT_Z = 2.  z is bit-identical
+                               either way.                                  */
   SPH_OPT_SAMPLER = 8       /* the draw of sph_fuse_sample at temperature > 0:
                                0 inverse CDF (default), 1 Gumbel-max: the
                                first index j of the largest

@@ -16,8 +16,7 @@ thread_local long long launch_count = 0;
 }
 
 namespace {
-constexpr int64_t kTcMinRows = 4;              // SPH_OPT_TC_MIN_ROWS
-constexpr long long kFinishWait = 1ll << 15;   // SPH_OPT_TC_FINISH_WAIT
+constexpr int64_t kTcMinRows = 4;              // SPH_OPT_TC_MIN_ROWS, the few-row kernel's fewest
 }
 
 struct ProfPair {
@@ -40,7 +39,7 @@ struct sph_ctx {
   int tc_block_k = 0;               // SPH_OPT_TC_BLOCK_K
   int tc_max_bn = 0;                // SPH_OPT_TC_MAX_BN
   int tc_tile_m = 0;                // SPH_OPT_TC_TILE_M
-  long long tc_finish_wait = kFinishWait;   // SPH_OPT_TC_FINISH_WAIT
+  long long tc_finish_wait = 1ll << 15;   // SPH_OPT_TC_FINISH_WAIT
   int sampler = 0;                  // SPH_OPT_SAMPLER
   int check_ids = 0;                // SPH_OPT_CHECK_IDS
   int split_quantize = 0;           // SPH_OPT_SPLIT_QUANTIZE
@@ -48,6 +47,7 @@ struct sph_ctx {
   int endpoint_z = 0;               // SPH_OPT_ENDPOINT_Z: 0 automatic, 1 store, 2 recompute
   int endpoint_rm = 0;              // SPH_OPT_ENDPOINT_ROWS_M: 0 automatic, 1 always, 2 never
   int gemv_quantize = 0;            // SPH_OPT_GEMV_QUANTIZE: 0 automatic, 1 never
+  bool few_never = false;           // SPH_OPT_FEW_ROWS: 0 automatic, 1 never
   // the cloud GEMV's last-block quantization: row maxima [8] and the
   // arrival ticket, zero between calls (the last block resets them)
   unsigned* gemv_q = nullptr;
@@ -158,14 +158,13 @@ int pair_mode(const sph_ctx* ctx) {
   return ctx->tc_pair == 1 ? 2 : 1;
 }
 
-// The tensor-core kernel's options all at their defaults: an explicit
-// crossover, schedule, tile, pair mode or z choice asks for the general
-// kernel, whose choices they are.
-bool default_tc_options(const sph_ctx* ctx) {
-  return ctx->tc_min_rows == kTcMinRows && ctx->tc_schedule == 0 && ctx->tc_stages == 0 &&
+// No option asks for the general tensor-core kernel: SPH_OPT_FEW_ROWS, or one
+// that shapes that kernel and means nothing to the few-row one.  (The others
+// hold there too: no pairs, no rows as M, no split tiles to finish.)
+bool few_allowed(const sph_ctx* ctx) {
+  return !ctx->few_never && ctx->tc_schedule == 0 && ctx->tc_stages == 0 &&
          ctx->tc_block_k == 0 && ctx->tc_max_bn == 0 && ctx->tc_tile_m == 0 &&
-         ctx->tc_finish_wait == kFinishWait && ctx->tc_pair == 0 && ctx->endpoint_rm == 0 &&
-         ctx->endpoint_z != 2;
+         ctx->tc_pair != 1 && ctx->endpoint_z != 2;
 }
 // Whether an endpoint contraction takes the few-row kernel, and its plan on
 // sm_count SMs: 4..32 rows over at most 512 columns, where the general
@@ -180,8 +179,8 @@ bool default_tc_options(const sph_ctx* ctx) {
 // little less, and it stays.
 bool few_shape(const sph_ctx* ctx, int64_t rows, int64_t n, int64_t K, bool gather, int sm_count,
                sph::FewPlan* pl) {
-  if (rows < ctx->tc_min_rows || rows > sph::kFewMaxRows || K > sph::kFewMaxK ||
-      !default_tc_options(ctx))
+  if (rows < ctx->tc_min_rows || rows < kTcMinRows || rows > sph::kFewMaxRows ||
+      K > sph::kFewMaxK || !few_allowed(ctx))
     return false;
   if (!sph::tc_plan((int)rows, (int)n, (int)K, 0, sm_count, 1, 0, 0, 0, gather, 0, 0, 0,
                     pair_mode(ctx), ctx->pair_units, 0)
@@ -822,6 +821,10 @@ sph_status sph_set_option(sph_ctx* ctx, sph_option option, int64_t value) {
     case SPH_OPT_CHECK_IDS:
       if (value != 0 && value != 1) return fail(ctx, SPH_ERR_INVALID_ARG, "check_ids must be 0 or 1");
       ctx->check_ids = (int)value;
+      return SPH_OK;
+    case SPH_OPT_FEW_ROWS:
+      if (value != 0 && value != 1) return fail(ctx, SPH_ERR_INVALID_ARG, "few_rows must be 0 or 1");
+      ctx->few_never = value == 1;
       return SPH_OK;
     case SPH_OPT_GEMV_QUANTIZE:
       if (value != 0 && value != 1) return fail(ctx, SPH_ERR_INVALID_ARG, "gemv_quantize must be 0 or 1");

@@ -23,13 +23,47 @@ def ctx():
 
 
 def general(ctx, f):
-    """f() on the general kernel (an explicit option asks for it)."""
+    """f() on the general kernel."""
     from paper_2607_13093_gb300 import sph
-    ctx.set_option(sph.SPH_OPT_TC_FINISH_WAIT, (1 << 15) - 1)
+    ctx.set_option(sph.SPH_OPT_FEW_ROWS, 1)
     try:
         return f()
     finally:
-        ctx.set_option(sph.SPH_OPT_TC_FINISH_WAIT, 1 << 15)
+        ctx.set_option(sph.SPH_OPT_FEW_ROWS, 0)
+
+
+def z_launches(ctx, w):
+    z = torch.empty(w.rows, w.n_keep, device=DEV)
+    ctx.profile_enable(True)
+    ctx.fuse_sample(None, None, w.h_local, w.W_l, keep_ids=w.keep_ids, draw=False,
+                    fused_logits_out=z)
+    ctx.sync()
+    n = ctx.profile_read()["launches"]
+    ctx.profile_enable(False)
+    return n
+
+
+# options of other calls and kernels leave the kernel to it; those that shape
+# the general one choose that (name, value, default, few-row kernel or not)
+@pytest.mark.parametrize("name,value,default,few", [
+    ("FEW_ROWS", 0, 0, True), ("TC_FINISH_WAIT", 0, 1 << 15, True), ("TC_MIN_ROWS", 1, 4, True),
+    ("TC_MIN_ROWS", 16, 4, True), ("TC_PAIR", 2, 0, True), ("ENDPOINT_ROWS_M", 1, 0, True),
+    ("ENDPOINT_Z", 1, 0, True), ("FEW_ROWS", 1, 0, False), ("TC_STAGES", 3, 0, False),
+    ("TC_SCHEDULE", 1, 0, False), ("TC_BLOCK_K", 64, 0, False), ("TC_MAX_BN", 16, 0, False),
+    ("TC_TILE_M", 128, 0, False), ("TC_PAIR", 1, 0, False), ("ENDPOINT_Z", 2, 0, False)])
+def test_which_options_choose_the_general_kernel(ctx, name, value, default, few):
+    from paper_2607_13093_gb300 import sph
+    opt = getattr(sph, "SPH_OPT_" + name)
+    ctx.set_option(opt, value)
+    try:
+        got = ctx.plan(1, 16, 12000, 256)["tile_ids"]
+    finally:
+        ctx.set_option(opt, default)
+    # 12000 ids: 125 tiles of 96 in one turn of the SMs; the general kernel's
+    # tiles have 128 or 256
+    assert (got == 96) if few else got in (128, 256)
+    with pytest.raises(sph.SphError):
+        ctx.set_option(sph.SPH_OPT_FEW_ROWS, 2)
 
 
 # rows (4, both sides of 16, 32), kept ids (segments, tiles and SM turns: one
@@ -49,7 +83,6 @@ def test_few_rows(ctx, rows, n, K, payload):
         Wp = torch.full((V, (K + 7) // 8 * 8), float("nan"), dtype=torch.bfloat16, device=DEV)
         Wp[:, :K] = w.W_l
         w.W_l = Wp[:, :K]
-    assert ctx.plan(1, rows, n, K)["block_rows"] in (16, 32)
     pc, ps = wl.make_payload(rows, n, seed=3, device=DEV) if payload else (None, None)
 
     def run():
@@ -63,6 +96,8 @@ def test_few_rows(ctx, rows, n, K, payload):
         ctx.sync()
         return z, t, g, y
 
+    # one launch for z alone on this kernel, two (operand split) on the general
+    assert z_launches(ctx, w) == 1 and general(ctx, lambda: z_launches(ctx, w)) == 2
     a, b = run(), general(ctx, run)
     for x, y in zip(a, b):
         assert torch.equal(x, y)
