@@ -182,8 +182,17 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const FewParams p) {
     s_abort = 1;
   };
 
+  // (a poll may suspend the thread for longer than this kernel's waits take,
+  // so the limit is looked at before each)
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    if (ptx::mbar_test(bar, parity)) return true;
+    const long long t0 = clock64();
+    while (clock64() - t0 < limit)
+      if (ptx::mbar_try_wait(bar, parity)) return true;
+    return false;
+  };
   auto warp_wait = [&](uint64_t* bar, uint32_t parity) {
-    const bool ok = __all_sync(0xFFFFFFFFu, !s_abort && ptx::mbar_wait(bar, parity, limit));
+    const bool ok = __all_sync(0xFFFFFFFFu, !s_abort && wait(bar, parity));
     if (!ok && lane == 0 && !s_abort) give_up();
     return ok;
   };

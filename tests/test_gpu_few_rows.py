@@ -124,13 +124,12 @@ def test_few_rows_one_call(ctx, rows, n, chunk):
             assert torch.equal(x, y)
 
 
-def test_few_rows_with_a_one_cycle_wait_limit(ctx):
-    # this kernel's waits are short enough that a polled barrier's own grace
-    # usually covers them, so a limit of one cycle may or may not run out:
-    # either the timeout is reported, or the call's logits are right; the
-    # context goes on in both cases
+@pytest.mark.parametrize("rows,n,K", [(4, 700, 48), (32, 30000, 256), (12, 44999, 512)])
+def test_few_rows_wait_timeout_is_reported_and_context_recovers(ctx, rows, n, K):
+    # with a limit of one cycle a wait is looked at once: the MMA warp's for
+    # the hidden states, which are still on their way from memory, gives up
     from paper_2607_13093_gb300 import sph
-    w = wl.make_workload(V=60000, d=264, d_l=256, rows=32, n_keep=30000, device=DEV, seed=93)
+    w = wl.make_workload(V=n + n // 3, d=K + 8, d_l=K, rows=rows, n_keep=n, device=DEV, seed=93)
     pc, ps = wl.make_payload(w.rows, w.n_keep, seed=3, device=DEV)
     z = torch.empty(w.rows, w.n_keep, device=DEV)
 
@@ -144,9 +143,9 @@ def test_few_rows_with_a_one_cycle_wait_limit(ctx):
     for _ in range(5):
         ctx.set_option(sph.SPH_OPT_SPIN_LIMIT, 1)
         try:
-            assert torch.equal(fuse(), want)
-        except sph.SphError as err:
-            assert err.status == 4, str(err)
+            with pytest.raises(sph.SphError) as err:
+                fuse()
         finally:
             ctx.set_option(sph.SPH_OPT_SPIN_LIMIT, 1 << 34)
+        assert err.value.status == 4, str(err.value)
         assert torch.equal(fuse(), want)
