@@ -16,7 +16,10 @@ between two uses of the same copy exceed twice the L2 size.
 
 Under torchrun every rank runs its own batch on its own GPU (independent
 sessions, weak scaling); the only collectives are the barrier and the
-max-over-ranks of the timed region.  Rank 0 prints one JSON line.
+max-over-ranks of the timed region.  Rank 0 prints one JSON line, short
+enough (LINE_BYTES) that whoever keeps only the end of the output keeps it
+whole; the notes, spreads and the block of the other workloads go to stderr as
+one JSON line before it.
 """
 from __future__ import annotations
 
@@ -69,6 +72,25 @@ def max_over_ranks(x, device=None):
 def job_rows_per_s(rows_per_rank, world, steps, ms):
     """Whole-job throughput: every rank's rows over the slowest rank's time."""
     return rows_per_rank * world * steps / (ms / 1e3)
+
+
+# The printed line: everything measured of its own workload but the long
+# notes; of these entries only the keys listed.
+LINE_BYTES = 2600
+LINE_OMITS = ("configs", "payload", "breakdown_note", "timed_loop")
+LINE_KEYS = {"roofline": ("bound", "achieved", "peak", "unit", "frac", "issued_frac", "kernel",
+                          "algorithmic_bytes", "algorithmic_flops", "traffic", "avg_launch_ms",
+                          "peak_source"),
+             "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps"),
+             "clocks": ("sm_mhz", "sm_max_mhz", "reasons", "samples"),
+             "cpu_baseline": ("value", "unit", "kind", "cores", "sample")}
+
+
+def line_of(out):
+    """The short line of a run's full record."""
+    def pick(k, v):
+        return {q: v[q] for q in LINE_KEYS[k] if q in v} if k in LINE_KEYS and v else v
+    return {k: pick(k, v) for k, v in out.items() if k not in LINE_OMITS}
 
 
 def parse():
@@ -910,7 +932,8 @@ def run_ours(args):
                                         args.config_cpu_seconds, with_cpu=with_cpu,
                                         mode=mode, chunk=chunk))
         out["configs"] = entries
-    print(json.dumps(out), flush=True)
+    print(json.dumps(out), file=sys.stderr, flush=True)
+    print(json.dumps(line_of(out)), flush=True)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()

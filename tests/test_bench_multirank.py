@@ -86,6 +86,46 @@ def test_reference_arm_under_torchrun_prints_once_from_rank_zero():
         assert key in out
 
 
+def test_the_printed_line_is_short_and_complete():
+    # a full record as a run makes it, with the block of the other workloads
+    # and every note: the line keeps the measured keys and stays below the
+    # 3000 bytes of output that are kept of a run
+    import json
+    import bench
+    note = "x" * 400
+    out = {
+        "metric": bench.METRIC, "value": 312345.6, "unit": bench.UNIT, "n_gpus": 1, "steps": 200,
+        "warmup": 50, "ms_per_step": 3.28549, "higher_is_better": True, "scaling": "weak",
+        "vs_baseline": None, "dtype": "f32", "data": "synthetic " + "x" * 66,
+        "config": {"workload": "w" * 160, "l2": "l" * 120, "rest": "r" * 260},
+        "breakdown_ms_per_step": {k: 2.57465 for k in "abcdef"}, "breakdown_note": note,
+        "roofline": {"bound": "tensor", "achieved": 830.18, "peak": 1890.3, "unit": "TFLOP/s",
+                     "frac": 0.4392, "issued_frac": 0.8784, "algorithmic_bytes": 2641342464,
+                     "algorithmic_flops": 2415919104000, "hbm": {"peak_note": note},
+                     "tensor": {"peak_note": note}, "avg_launch_ms": 2.9101, "traffic": 5535950000,
+                     "kernel": "k" * 90, "timing": note, "spread": {"note": note},
+                     "peak_source": "measured (MEASURED_PEAKS.json)"},
+        "gpu_launches": 1200, "timed_loop": note, "payload": {"what": note},
+        "e2e": {"value": 299941.3, "unit": "rows/s", "h2d_bytes_per_step": 20971520,
+                "d2h_bytes_per_step": 4096, "steps": 200, "direct_calls": {"value": 1.0},
+                "note": note},
+        "clocks": {"sm_mhz": 1597.0, "sm_max_mhz": 2070.0, "reasons": ["sw_power_cap"],
+                   "samples": 13, "note": note},
+        "cpu_baseline": {"value": 0.6366084836307984, "unit": "rows/s", "cores": 16,
+                         "kind": "oracle", "sample": "s" * 110, "seconds": 12.17},
+        "configs": [{"workload": note}] * 30}
+    line = bench.line_of(out)
+    assert len(json.dumps(line)) <= bench.LINE_BYTES < 3000
+    assert not set(line) & set(bench.LINE_OMITS)
+    for k, v in out.items():
+        if k not in bench.LINE_OMITS and k not in bench.LINE_KEYS:
+            assert line[k] == v
+    assert set(line["e2e"]) >= {"value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"}
+    assert set(line["clocks"]) >= {"sm_mhz", "sm_max_mhz", "reasons"}
+    assert line["roofline"]["traffic"] == 5535950000
+    assert bench.line_of(dict(out, clocks=None))["clocks"] is None
+
+
 def test_traffic_record_follows_its_own_sources(tmp_path, monkeypatch):
     # a committed DRAM-traffic record counts while the kernel sources it
     # lists hash as they did when it was taken, and is dropped once one of
