@@ -1183,14 +1183,6 @@ tc_kernel(const __grid_constant__ WMaps wm,
       constexpr int kMaxC = 8;
       int c0 = 0, C = 1, cnt = 0;
       bool fin = false, known_last = false;
-      // two or three contributors: the others' partials of the next chunk
-      // (the finisher is the last but one, so pa comes before and pb after
-      // its own part with three, pa after it with two)
-      // (the endpoint's epilogues have no registers for them: with them the
-      // per-lane form spilled 250 bytes, and 32 rows x 12000 ids x 4096 took
-      // 41.9 us instead of 36.0)
-      constexpr bool kParts = EPI == EPI_CLOUD;
-      float pa[kParts ? 16 : 1], pb[kParts ? 16 : 1];
       if (!whole) {
         cnt = ((tile * 4 + quad) * kEpiGroups + grp) * (PAIR ? 2 : 1) + half;
         c0 = (int)cta_of((long long)tile * p.KB, p.T, G);
@@ -1208,33 +1200,6 @@ tc_kernel(const __grid_constant__ WMaps wm,
       auto slot_of = [&](int c) {
         return pslot(c == 0 ? 2 * c0 + (c0_first ? 0 : 1) : 2 * (c0 + c));
       };
-      if (fin) {
-        // the early contributor (the tile's last) has usually arrived
-        // already: then fetch its partial while the MMAs finish
-        int arrived = 0;
-        if (lane == 0) arrived = ptx::ld_acquire_gpu(&p.counters[cnt]);
-        known_last = __shfl_sync(0xFFFFFFFFu, arrived, 0) == C - 1;
-        __syncwarp();
-      }
-      auto load_parts = [&](int hc) {
-        const int hf = hc / nch, ch = hc - hf * nch;
-        const size_t o = (size_t)ch * 16 * TM + hf * 128 + quad * 32 + lane;
-        if constexpr (kParts) {
-          const float* p0 = p.P + (size_t)slot_of(C == 2 ? 1 : 0) * BN * TM + o;
-#pragma unroll
-          for (int q = 0; q < 16; ++q) pa[q] = __ldcg(p0 + q * TM);
-          if (C == 3) {
-            const float* p1 = p.P + (size_t)slot_of(2) * BN * TM + o;
-#pragma unroll
-            for (int q = 0; q < 16; ++q) pb[q] = __ldcg(p1 + q * TM);
-          }
-        }
-      };
-      // (arrived before the accumulator is ready: the first chunk's are
-      // fetched while the MMAs finish)
-      const bool parts = kParts && (C == 2 || C == 3);
-      bool pre_ok = known_last && parts && grp < nhc;
-      if (pre_ok) load_parts(grp);
       int ok = 1;
       if (lane == 0)
         ok = !*s_abort && ptx::mbar_wait(&tfull[acc], fph[acc], limit);
@@ -1244,7 +1209,7 @@ tc_kernel(const __grid_constant__ WMaps wm,
         break;
       }
       fph[acc] ^= 1;
-      if (fin && !known_last) {
+      if (fin) {
         // the other contributors that end with this tile finish at about
         // the same time: poll for them, bounded (giving up only costs the
         // round trip through the partial buffer)
@@ -1259,7 +1224,6 @@ tc_kernel(const __grid_constant__ WMaps wm,
         known_last = __shfl_sync(0xFFFFFFFFu, arrived, 0) == C - 1;
         __syncwarp();
       }
-      if (known_last && parts && !pre_ok && grp < nhc) load_parts(grp);
       ptx::tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) +
                              (uint32_t)(acc * kHalves * BN);
@@ -1278,20 +1242,7 @@ tc_kernel(const __grid_constant__ WMaps wm,
           finish_rm<EPI, kU>(p, v1, r_rm, t * 256 + s1 * 32, rp[a + 1], rq_rm);
         }
       }
-      // a split tile of two or three contributors: its partials a chunk ahead
-      const bool by_parts = known_last && parts;
-      if constexpr (kParts) {
-        for (int hc = grp; hc < (by_parts ? nhc : 0); hc += kEpiGroups) {
-          const int hf = hc / nch, ch = hc - hf * nch;
-          float v[16];
-          ptx::tmem_ld16(taddr + hf * BN + ch * 16, v);
-#pragma unroll
-          for (int q = 0; q < 16; ++q) v[q] = C == 2 ? v[q] + pa[q] : (pa[q] + v[q]) + pb[q];
-          if (hc + kEpiGroups < nhc) load_parts(hc + kEpiGroups);
-          finish(v, hf, ch);
-        }
-      }
-      for (int hc = grp; hc < (rm || by_parts ? 0 : nhc); hc += kEpiGroups) {
+      for (int hc = grp; hc < (rm ? 0 : nhc); hc += kEpiGroups) {
         const int hf = hc / nch, ch = hc - hf * nch;
         const int i = hf * 128 + quad * 32 + lane;
         float v[16];
@@ -1316,6 +1267,10 @@ tc_kernel(const __grid_constant__ WMaps wm,
         } else if (known_last) {
           // the partials in CTA order (the same order, and so the same
           // result, as the fix-up below), this CTA's own from registers
+          // (fetched here, not a chunk ahead: with 16 or 32 registers of them
+          // ahead the cloud call of 487 rows x 872 ids x 3840 took 59.9 us
+          // instead of 58.0, 32 x 12000 x 3840 30.7 instead of 30.5, and the
+          // per-lane endpoint spilled)
           if constexpr (lane_pay) load_payload<EPI>(p, rb * BN + ch * 16, J(hf), lane, pay);
           const int me = unit - c0;
           const size_t o = (size_t)ch * 16 * TM + i;
