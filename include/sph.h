@@ -208,7 +208,9 @@ typedef enum sph_option {
                                0 automatic (default: for 4..32 rows, from
                                SPH_OPT_TC_MIN_ROWS on, over d_l <= 512, where
                                the general tensor-core kernel would take
-                               whole tiles too), 1 never.  The options that
+                               whole tiles too and, above d_l = 384, for at
+                               most three 128-id tiles an SM or at most 16
+                               rows of a subset), 1 never.  The options that
                                shape the general kernel ask for it as well:
                                any SPH_OPT_TC_SCHEDULE, _STAGES, _BLOCK_K,
                                _MAX_BN or _TILE_M but 0, SPH_OPT_TC_PAIR = 1

@@ -169,14 +169,20 @@ bool few_allowed(const sph_ctx* ctx) {
 // Whether an endpoint contraction takes the few-row kernel, and its plan on
 // sm_count SMs: 4..32 rows over at most 512 columns, where the general
 // kernel would take whole tiles as well.  Endpoint call with its draw,
-// general against few-row kernel, us: 32 rows x 12000 ids x 256 13.3 / 9.9,
-// x 60000 x 96 25.4 / 16.9, x 256000 x 512 83.4 / 77.7; 12 rows x 44999 x 512
-// 27.1 / 21.1; 4 rows x 700 x 48 11.0 / 7.1.  Past 512 columns the copies'
-// arrivals weigh more than the launch and the set-up saved (32 rows x 60000 x
-// 1024 43.9 / 51.3, 24 x 152064 x 1024 79.8 / 89.7).  Over whole tiles both
-// kernels add in the same order, so z has the same bits; where the general
-// kernel would split a tile's columns over CTAs its shorter chains round a
-// little less, and it stays.
+// general / few-row kernel, us: 4 rows x 700 ids x 48 10.9 / 7.9; 32 rows x
+// 12000 x 256 12.7 / 9.8, x 60000 x 96 22.3 / 15.4, x 152064 x 256 39.4 / 33.4;
+// 12 rows x 44999 x 512 23.9 / 21.0.  A stage of columns costs this kernel
+// more (its copies arrive thread by thread) and a call less, so past 384
+// columns it depends: up to three turns of the SMs it wins (32 rows x 12000 x
+// 512 14.1 / 12.3, x 51302 25.5 / 23.9), beyond them only with at most 16 rows
+// whose ids are gathered (12 rows x 100000 of 152064 x 512 37.7 / 33.5, but 32
+// rows x 128000 of 256000 42.9 / 44.6, and over a full vocabulary, which the
+// general kernel copies in one piece, 4 x 152064 40.3 / 41.9, 32 x 256000
+// 66.9 / 73.7).  Past 512 a short call still gains (12 rows x 12000 x 768 15.8 /
+// 13.9) and a long one does not (32 x 152064 x 640 50.4 / 56.0); the line stays
+// where both are near.  Over whole tiles both kernels add in the same order,
+// so z has the same bits; where the general kernel would split a tile's
+// columns over CTAs its shorter chains round a little less, and it stays.
 bool few_shape(const sph_ctx* ctx, int64_t rows, int64_t n, int64_t K, bool gather, int sm_count,
                sph::FewPlan* pl) {
   if (rows < ctx->tc_min_rows || rows < kTcMinRows || rows > sph::kFewMaxRows ||
@@ -187,6 +193,7 @@ bool few_shape(const sph_ctx* ctx, int64_t rows, int64_t n, int64_t K, bool gath
            .whole_tiles)
     return false;
   *pl = sph::few_plan((int)rows, (int)n, (int)K, sm_count);
+  if (K > 384 && pl->tiles > 3 * sm_count && (rows > 16 || !gather)) return false;
   return pl->ok;
 }
 bool few_route(const sph_ctx* ctx, const sph::GatherGemm& g, int sm_count, sph::FewPlan* pl) {

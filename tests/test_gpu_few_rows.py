@@ -66,6 +66,19 @@ def test_which_options_choose_the_general_kernel(ctx, name, value, default, few)
         ctx.set_option(sph.SPH_OPT_FEW_ROWS, 2)
 
 
+@pytest.mark.parametrize("rows,n,V,K,few", [
+    (32, 58368, 70000, 512, True),                   # 456 tiles: three an SM
+    (32, 58369, 70000, 512, False), (17, 77824, 90000, 392, False), (16, 77824, 90000, 392, True),
+    (16, 77824, 77824, 392, False), (32, 77824, 77824, 384, True), (12, 45000, 45000, 512, True),
+    (4, 77824, 90000, 520, False)])
+def test_the_lines_over_long_hidden_dimensions(ctx, rows, n, V, K, few):
+    # three turns of the 152 SMs, 16 rows, a subset or the full vocabulary
+    w = wl.make_workload(V=V, d=K + 8, d_l=K, rows=rows, n_keep=n, seed=n, device=DEV)
+    assert (w.keep_ids is None) == (n == V)
+    g = general(ctx, lambda: ctx.plan(1, rows, n, K, gather=n < V))
+    assert (z_launches(ctx, w) == 1) == (few and g["whole_tiles"] == 1)
+
+
 # rows (4, both sides of 16, 32), kept ids (segments, tiles and SM turns: one
 # turn of 152 tiles ends at 19456 ids), columns (atoms of 64, stages of 128)
 CASES = [(4, 1, 48), (5, 31, 8), (16, 33, 64), (17, 128, 65), (32, 129, 128), (31, 700, 96),
