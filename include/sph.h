@@ -155,10 +155,10 @@ typedef enum sph_option {
                                loading 128 ids of the weights and half of the
                                hidden-state rows.  0 (default): where the row
                                blocks are long (cloud: >= 128 rows with bf16
-                               weights; with e4m3 weights >= 224, or >= 160
-                               for bf16-rounded activations, where whole
-                               tiles are scheduled either way; endpoint:
-                               >= 192);
+                               weights; with e4m3 weights >= 224, or one
+                               block of >= 192, or of >= 160 for bf16-rounded
+                               activations, where whole tiles are scheduled
+                               either way; endpoint: >= 192);
                                1: always (SPH_ERR_UNSUPPORTED where pairs
                                cannot be scheduled);
                                2: never.  The results are the fp32 sums of

@@ -1891,14 +1891,19 @@ TcPlan tc_plan(int rows, int n, int K, int act_bf16, int sm_count, int endpoint,
   pl.ok = pl.stages >= 2;
   // e4m3 weights on pairs, whose row blocks pass the 128 rows of a single CTA
   // (its MMAs of N = 128 read 8 KB of operands in 64 cycles, all that shared
-  // memory gives, beside the copies).  Cloud call, single / pair us: four
-  // planes, 256 rows x 152064 x 7168 752 / 700, 512 x 64000 x 3584 336 / 321,
-  // 1024 x 32000 x 3584 366 / 353, but 300 rows (160-row blocks) x 152064 x
-  // 4608 644 / 733; two planes, 256 rows x 152064 x 7168 432 / 405, 130 rows
-  // 319 / 310.  Where both plans take whole tiles: their sums have the same
-  // bits.
-  if (fp8 && pp.pair && pp.ok && pp.BN >= (pl.hilo == 4 ? 224 : 160) && pp.whole_tiles &&
-      pl.whole_tiles)
+  // memory gives, beside the copies): in one block from 192 rows with four
+  // planes and from 160 with two, against two short blocks of single CTAs, and
+  // in several from 224, against blocks of up to 128.  Cloud call, single /
+  // pair us: four planes, 190 rows x 152064 x 7168 657 / 575, 224 699 / 632, 256
+  // 738 / 692, 512 x 64000 x 3584 322 / 299; below, in blocks of 160 and 192, 300
+  // rows x 152064 x 7168 960 / 1017, 380 x 64000 x 3584 239 / 256.  Two planes,
+  // 130 rows x 152064 x 7168 313 / 274, 190 353 / 322, 400 734 / 657, 440 x 64000 x
+  // 3584 178 / 158; below, 280 x 64000 x 3584 126 / 135, 320 x 128000 x 1024 133 /
+  // 143, 350 x 64000 x 3584 140 / 149 (but 380 x 152064 x 7168 647 / 615).  Where
+  // both plans take whole tiles: their sums have the same bits (four planes in
+  // blocks of 160 would put two atoms in a stage, and add in another order).
+  if (fp8 && pp.pair && pp.ok && pp.whole_tiles && pl.whole_tiles &&
+      pp.BN >= (pp.RB > 1 ? 224 : pl.hilo == 4 ? 192 : 160))
     return pp;
   return pl;
 }

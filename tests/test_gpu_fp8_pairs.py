@@ -11,10 +11,26 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
+# one block of 160 or 192 rows, two of 160, 192 and 224, on whole tiles
+@pytest.mark.parametrize("rows,four,two", [(128, 0, 0), (130, 0, 1), (160, 0, 1), (161, 1, 1),
+                                           (192, 1, 1), (256, 1, 1), (257, 0, 0), (384, 0, 0),
+                                           (385, 1, 1), (1024, 1, 1)])
+def test_which_row_blocks_pair(rows, four, two):
+    from paper_2607_13093_gb300 import build_lib
+    build_lib.build()
+    from paper_2607_13093_gb300 import sph
+    ctx = sph.Context(0)
+    for act, pair in ((sph.SPH_ACT_FP32, four), (sph.SPH_ACT_BF16, two)):
+        p = ctx.plan(0, rows, 152064, 7168, w_dtype=sph.SPH_DTYPE_FP8_E4M3, act_mode=act,
+                     gather=False)
+        assert p["whole_tiles"] == 1 and p["pair"] == pair
+    ctx.close()
+
+
 # rows (one 256-row block short of, at and past its end), kept ids (256-id
 # tiles: short, ragged, whole), hidden columns (128-column blocks, ragged)
 @pytest.mark.parametrize("rows,keep,d_h", [(225, 3000, 256), (256, 2999, 1008), (250, 257, 128),
-                                           (480, 700, 400), (513, 1100, 1024)])
+                                           (480, 700, 400), (513, 1100, 1024), (190, 1500, 528)])
 @pytest.mark.parametrize("act", ["fp32", "bf16"])
 def test_wide_row_blocks_on_pairs(rows, keep, d_h, act):
     from paper_2607_13093_gb300 import build_lib
