@@ -14,8 +14,8 @@
 //   A   the tile's weight rows by 16-byte cp.async with per-thread row
 //       pointers: any id pattern costs the same, and the first copies go out
 //       as soon as the ids are there (where kernels of the same call ran
-//       before this one: before it waits for them).  Rows past the tile hold stale bytes
-//       and land in accumulator lanes that are never read.
+//       before this one: before it waits for them).  Rows past the tile hold
+//       stale bytes and land in accumulator lanes that are never read.
 //   D   fp32 in TMEM, two tiles' accumulators.  Every 64 columns multiply hi,
 //       then lo, in the order of the general kernel, so z has the same bits.
 //
@@ -26,11 +26,11 @@
 // landed.
 //
 // What bounds it: launch, set-up and one round trip each for ids, weights and
-// payload (4 rows x 700 ids x 48 columns with its draw: 7.1 us, general
-// kernel 11.0); past that the epilogues (32 rows x 60000 ids x 96: 16.9 us,
-// 25.4) and, at 512 columns, the copies: they arrive on a stage's barrier
-// thread by thread, about 600 cycles a stage (12 rows x 44999 ids x 512: 21.1
-// us, 27.1).  A long hidden dimension would pay that at every stage, so the
+// payload (4 rows x 700 ids x 48 columns with its draw: 7.9 us, general
+// kernel 10.9); past that the epilogues (32 rows x 60000 ids x 96: 15.4 us,
+// 22.3) and, at 512 columns, the copies: they arrive on a stage's barrier
+// thread by thread, about 600 cycles a stage (12 rows x 44999 ids x 512: 21.0
+// us, 23.9).  A long hidden dimension would pay that at every stage, so the
 // general kernel's tensor copies keep those (an earlier form of this kernel
 // for 3840 columns: 35 us against 28).
 #include <atomic>

@@ -581,7 +581,9 @@ __device__ __forceinline__ float2 chunk_segment_stats(const float* z, int left,
 // memory.  Token calls of d_l 64 with it and without: 1 row x 2048 ids 5.5 us
 // and 6.7, 3 x 8192 9.8 and 11.4, 16 x 8192 21.4 and 23.0.  A chunk a warp at
 // most: with two, 3 x 16382 ids took 14.8 us instead of 14.6.  16 rows at
-// most: 300 x 2048 took 193 us instead of 174.
+// most: a row is one block here, and with more rows the gain is a launch's and
+// fades (20 x 2048 ids 15.7 us and 17.2, 64 x 8192 73.6 and 75.0, 128 x 2048 81.6
+// and 76.4); above 3 rows the GEMV runs only where the crossover is raised.
 constexpr int kShortChunks = kWarps;
 constexpr int kShortRows = 16;
 __global__ void __launch_bounds__(kWarps * 32)

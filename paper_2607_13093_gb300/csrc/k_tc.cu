@@ -78,15 +78,17 @@ constexpr float kLog2eF = 1.4426950408889634f;   // exp(d / tau) = 2^(d log2(e) 
 // Kernel instantiations of EPI_ENDPOINT that finish through the per-warp
 // shared-memory transpose (finish_chunk_t) rather than per lane.
 constexpr int EPI_ENDPOINT_T = 3;
-// The two forms of the transposed and (below) the rows-as-M endpoint whose
-// rows of codes start anywhere: the codes are fetched as the aligned words
-// that hold them, one more than the aligned forms need, and put together only
-// where they are used.  (Assembling them at the load, from whatever narrower
-// loads the alignment allows, made every chunk wait for memory, and cost the
-// rows-as-M form 32 scattered byte loads a segment: endpoint call with its
-// draw over 51302 ids x 512, 256 rows 54.8 -> 44.2 us, 512 rows 104.6 -> 70.9;
-// z alone for 320 rows 66.3 -> 62.9.  The extra registers cost the aligned
-// shapes up to 11 %, so these are instantiations of their own.)
+// The two forms of the transposed and (below) the rows-as-M endpoint for rows
+// of codes off the words that the aligned forms load (the transposed one at
+// even addresses, as everything it takes; rows as M at any): the codes are
+// fetched as the aligned words that hold them, one more than the aligned forms
+// need, and put together only where they are used.  (Assembled at the load,
+// from whatever narrower loads the alignment allows, they made every chunk wait
+// for memory, and cost the rows-as-M form 32 scattered byte loads a segment:
+// endpoint call with its draw over 51302 ids x 512, 256 rows 54.8 us and 44.2 as
+// words, 512 rows 104.6 and 70.9; z alone for 320 rows 66.3 and 58.6.  The extra
+// registers cost the aligned shapes up to 11 %, so these are instantiations of
+// their own.)
 constexpr int EPI_ENDPOINT_TU = 6;
 constexpr int EPI_ENDPOINT_RMU = 7;
 // Rows-as-M instantiations of EPI_ENDPOINT and EPI_FUSED (CTA pairs only):
@@ -242,10 +244,9 @@ __device__ __forceinline__ void prefetch_payload(const TcParams& p, int row0, in
 // A warp runs it alone on its scheduler or with one other, so its length is
 // its instructions' latency: chunks whose rows and ids all exist (nearly all)
 // take a path without a predicate and an address product per value (a cloud
-// chunk of few rows 2800 cycles with them, 1100 without; with the split tiles'
-// partials fetched a chunk ahead the decode step went from 43.5 to 42.9 us,
-// 32 rows x 60000 ids 114.9 -> 110.7, 320 x 51302 287.2 -> 273.7, unsplit 147 x
-// 32000 x 4096 95.3 -> 91.5).
+// chunk of few rows 2800 cycles with them, 1100 without; cloud call with and
+// without, 32 rows x 12000 ids x 3840 31.3 / 30.7 us, 320 x 51302 x 3584 183.2 /
+// 173.5, 300 x 3000 x 4096 47.3 / 43.8).
 template <int EPI>
 __device__ __forceinline__ void finish_chunk(const TcParams& p, const float (&v)[16],
                                              int row0, int j, bool vj, int id,

@@ -119,10 +119,12 @@ __device__ __forceinline__ void tc_fence_after() {
 // loop's counters, addresses and descriptors are then warp-uniform and stay
 // in the uniform registers that the instruction takes its operands from (a
 // loop run by a single lane moves each one there first: 75-100 cycles an MMA,
-// longer than a short MMA itself; steps before and after: 32 rows x 12000 ids
-// 44.4 -> 43.5 us, 32 x 60000 118.2 -> 114.9, the drafted 320 x 51302 293.9 ->
-// 287.2, 1024 x 256000 3367 -> 3317).  elect.sync elects the same lane every
-// time, so commits cover the MMAs.
+// longer than a short MMA itself; by one lane and by the warp: the step of 32
+// rows x 12000 ids 44.4 us and 43.5, 32 x 60000 118.2 and 114.9, the drafted 320 x
+// 51302 293.9 and 287.2).  So do the waits: polled by one lane they make the
+// loop divergent (cloud call of 32 rows x 12000 ids x 3840 37.8 us and 30.7, 320
+// x 51302 x 3584 272 and 173).  elect.sync elects the same lane every time, so
+// commits cover the MMAs.
 //
 // Shared-memory matrix descriptor: K-major operand stored as 8-row groups of
 // 128-byte rows with the 128-byte swizzle (the layout TMA's SWIZZLE_128B

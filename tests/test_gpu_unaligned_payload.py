@@ -1,7 +1,8 @@
-"""Payloads whose rows of codes start anywhere: the transposed and the
-rows-as-M endpoint fetch them as the aligned words that hold them.  The same
-bits for every base address, and the oracle's values.  Needs a GPU (marked
-gpu)."""
+"""Payloads whose rows of codes start anywhere: the transposed endpoint (rows at
+even addresses) and the rows-as-M one (at any) fetch them as the aligned words
+that hold them; rows at odd addresses with ids as M take the per-lane epilogue.
+The same bits for every base address, and the oracle's values.  Needs a GPU
+(marked gpu)."""
 import pytest
 import torch
 
@@ -12,8 +13,8 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-# 160 rows: ids as M through the transpose (an even number of ids); 250: rows
-# as M.  Ids: whole 32-id segments, and last segments of 1, 8, 10 and 31 ids;
+# 160 rows: ids as M, through the transpose at the even shifts (the number of
+# ids is even), lane by lane at the odd ones; 250: rows as M at all of them.  Ids: whole 32-id segments, and last segments of 1, 8, 10 and 31 ids;
 # divisible by 16, 8, 4, 2 and 1
 @pytest.mark.parametrize("rows,n", [(160, 1024), (160, 1032), (160, 1034), (160, 1036), (250, 1024),
                                     (250, 1032), (250, 1034), (250, 1055), (250, 1025)])
